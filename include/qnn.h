@@ -53,7 +53,9 @@ typedef enum {
 
 /* Convolution algorithm choice (qnn_conv_desc.algo). */
 enum {
-    QNN_ALGO_AUTO = 0,         /* tensor-core kernel when the shape allows it, else the CUDA-core kernel */
+    QNN_ALGO_AUTO = 0,         /* tensor-core kernel with preparable filters when the shape allows it, else a kernel
+                                  that needs no workspace (reported as QNN_ALGO_DIRECT: at INT-8 the tensor-core
+                                  gather kernel, else the CUDA-core kernel) */
     QNN_ALGO_DIRECT = 1,       /* CUDA-core kernel (dp4a), any stride / padding */
     QNN_ALGO_TENSORCORE = 2,   /* tcgen05 implicit GEMM (the window kernel when its plan fits, else the
                                   general one); QNN_EUNSUPPORTED when neither fits the shape */

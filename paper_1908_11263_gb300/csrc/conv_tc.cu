@@ -1233,8 +1233,12 @@ __global__ void __launch_bounds__(256) conv_tc_prep_kernel(const uint8_t *w, con
     const int taps = kh * kw;
     const int slot_of[8] = {0, 2, 4, 6, 1, 3, 5, 7};  // inverse of {0,4,1,5,2,6,3,7}
     int sum = 0, pos = 0, neg = 0;  // |sum| <= K * 2^(Q-1) < 2^31 (accumulator bound of the ABI)
-    for (int tap = 0; tap < taps; ++tap) {
-        for (int cc = lane; cc < c_pad; cc += 32) {  // consecutive lanes: consecutive channels and slots
+    // 64 channels at a time (the gather kernel's stages), all taps of them
+    for (int group = 0; group * 64 < c_pad; ++group) {
+      const int first_pos = pos, first_neg = neg;
+      for (int tap = 0; tap < taps; ++tap) {
+        for (int cc = group * 64 + lane; cc < min(c_pad, group * 64 + 64); cc += 32) {
+            // consecutive lanes: consecutive channels and slots
             int v = 0;
             if (o < m && cc < c) {
                 const long long e = (static_cast<long long>(o) * taps + tap) * c + cc;
@@ -1262,6 +1266,13 @@ __global__ void __launch_bounds__(256) conv_tc_prep_kernel(const uint8_t *w, con
                 wpack[dst] = __half_as_ushort(__int2half_rn(v));
             }
         }
+      }
+      if (nchunks == 0 && group < kThrStride) {  // the gather kernel: the group's sum of |w|
+          int abs = (pos - first_pos) - (neg - first_neg);
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) abs += __shfl_xor_sync(0xffffffffu, abs, d);
+          if (lane == 0) thr_out[o * kThrStride + group] = abs;
+      }
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
@@ -1542,8 +1553,10 @@ TcPlan plan_conv_tc(const ConvShape &s)
     return plan_layout(s, false);
 }
 
+size_t conv_tc_chan_offset(const TcPlan &plan) { return chan_offset(plan); }
+
 cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const ConvParams &p, void *workspace,
-                                cudaStream_t st)
+                                cudaStream_t st, int chunks)
 {
     uint16_t *wpack = static_cast<uint16_t *>(workspace);
     int4 *chan = reinterpret_cast<int4 *>(static_cast<uint8_t *>(workspace) + chan_offset(plan));
@@ -1552,7 +1565,7 @@ cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const Co
 #define QNN_PREP(B)                                                                                              \
     conv_tc_prep_kernel<B><<<(mp + 7) / 8, 256, 0, st>>>(p.w, p.bias, p.kappa, p.lambda, p.shifts, p.shift, s.m, \
                                                          mp, s.kh, s.kw, s.c, plan.c_pad, plan.k_pad, plan.nt,   \
-                                                         plan.nchunks, plan.fp8, wpack, chan, p.thresholds, thr)
+                                                         chunks, plan.fp8, wpack, chan, p.thresholds, thr)
     switch (s.bits) {
         case 8: QNN_PREP(8); break;
         case 4: QNN_PREP(4); break;

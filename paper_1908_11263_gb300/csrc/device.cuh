@@ -64,6 +64,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
     return ok != 0;
 }
 
+__device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Warp-collective bounded wait: every lane of a converged warp calls it and
 // every lane observes the phase completion itself (so each has the acquire
 // ordering of the barrier).  All lanes poll with try_wait, which parks them in
@@ -71,18 +84,26 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
 // the order of a hundred cycles, where a single polling lane, a sleep between
 // polls or a shuffle of the result each add more.  Returns false on every lane
 // (and records QNN_ETIMEOUT in *status) once `limit_cycles` SM cycles pass.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, int *status,
-                                               long long limit_cycles = kWaitLimitCycles)
+__device__ __forceinline__ bool mbar_wait_warp_at(uint32_t bar, uint32_t parity, int *status,
+                                                  long long limit_cycles = kWaitLimitCycles)
 {
+    // a phase that has completed already costs no clock read
+    if (__all_sync(0xffffffffu, mbar_try_wait_at(bar, parity))) return true;
     const long long t0 = clock64();
     while (true) {
-        const bool ok = mbar_try_wait(bar, parity);
+        const bool ok = mbar_try_wait_at(bar, parity);
         if (__all_sync(0xffffffffu, ok)) return true;
         if (__any_sync(0xffffffffu, clock64() - t0 > limit_cycles)) {
             if ((threadIdx.x & 31) == 0) report(status, QNN_ETIMEOUT);
             return false;
         }
     }
+}
+
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, int *status,
+                                               long long limit_cycles = kWaitLimitCycles)
+{
+    return mbar_wait_warp_at(smem_addr(bar), parity, status, limit_cycles);
 }
 
 // ------------------------------------------------------------------ bulk copy (TMA, untiled)
@@ -203,6 +224,15 @@ __device__ __forceinline__ void mma_f8_ss_warp_nc(uint32_t d_tmem, uint64_t a_de
         "setp.ne.b32 p, %4, 0;\n\t"
         "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+}
+
+__device__ __forceinline__ void mma_commit_warp_at(uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 __device__ __forceinline__ void mma_commit_warp(uint64_t *bar)

@@ -66,8 +66,13 @@ struct TcPlan {
 };
 
 TcPlan plan_conv_tc(const ConvShape &s);
+// chunks: accumulators per output whose pre-load the records remove
+// (plan.nchunks for conv_tc; 0 for the gather kernel, which has no pre-load and
+// gets the sums of |w| by filter and 64-channel group behind the records).
 cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const ConvParams &p, void *workspace,
-                                cudaStream_t st);
+                                cudaStream_t st, int chunks);
+// where launch_conv_tc_prep puts the compression records in the workspace
+size_t conv_tc_chan_offset(const TcPlan &plan);
 // after_prep: launched right after launch_conv_tc_prep on the same stream, so the
 // convolution may start while the preparation kernel still runs.
 cudaError_t launch_conv_tc_run(const TcPlan &plan, const ConvShape &s, const uint8_t *x, uint8_t *y,
@@ -117,6 +122,32 @@ cudaError_t launch_conv_win(const WinPlan &plan, const ConvShape &s, const ConvP
 // (plan.img_bytes) to `workspace`.
 cudaError_t prepare_conv_win(const WinPlan &plan, const ConvShape &s, const ConvParams &p, void *workspace,
                              cudaStream_t st);
+
+// ---- tensor-core gather kernel (INT-8, any stride, padding and alignment) -- conv_gather*
+struct GatherPlan {
+    bool ok;
+    int flat;                // flat window (stride 1, prepared filters), else im2col
+    int aligned;             // c a multiple of 16: aligned 16-byte granules
+    int gran_row;            // granules per kernel row
+    int taps, cgr, nxs;      // taps per pixel stage; granules per tap; stages per tile
+    int chunk_stages;        // stages per exact accumulator chunk, whatever the filters
+    int wp;                  // flat: positions per row
+    int npix;                // columns in all (im2col: output pixels; flat: positions)
+    int ncols, npos, mtiles; // columns per tile; staged positions; tiles
+    int w_rows, n_ntiles;    // filters per block as they are laid out; blocks
+    int mstep, grid;         // CTAs per block of filters; CTAs
+    int resident, parts;     // filters kept in shared memory, arriving in parts
+    int stages, w_slots, unrolled;
+    uint32_t plane_x, stage_bytes, plane_w, item_w, off_x, off_bar, smem_bytes;
+};
+
+// w_rows: filters per block of the workspace that launch_conv_tc_prep wrote
+// (with chunks = 0); 0: packed filters as the caller keeps them.
+GatherPlan plan_conv_gather(const ConvShape &s, int w_rows, int sms);
+cudaError_t launch_conv_gather(const GatherPlan &plan, const ConvShape &s, const ConvParams &p, cudaStream_t st);
+// wpack, chan: the filters and records launch_conv_tc_prep wrote
+cudaError_t launch_conv_gather_prepared(const GatherPlan &plan, const ConvShape &s, const uint8_t *x, uint8_t *y,
+                                        const void *wpack, const void *chan, cudaStream_t st);
 
 // ---- max-pool, fully connected, packing
 cudaError_t launch_maxpool(int n, int h, int w, int c, int k, int s, int bits, const uint8_t *x, uint8_t *y,
