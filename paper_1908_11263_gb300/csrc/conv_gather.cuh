@@ -877,25 +877,6 @@ __device__ __forceinline__ bool channel_record(const Args &a, Shared *sh, int nt
     return true;
 }
 
-// An accumulator (an integer of magnitude at most 2^24) as int32.  The
-// conversion unit takes 16 values a cycle per SM, an eighth of the rate of the
-// fp32 pipe, where the value can be split exactly instead: hi = rn(v / 2^12)
-// and v - 2^12 hi (at most 2^11), each brought to an integer by adding 1.5 * 2^23
-// (bits 0x4B400000).  12 of every 32 values take the one way, 20 the other
-// (580 cycles for 32 columns of a warp with the conversion unit alone).
-__device__ __forceinline__ int split_to_int(float v)
-{
-    const float magic = __uint_as_float(0x4B400000u);
-    const float t = fmaf(v, 1.0f / 4096.0f, magic);
-    const float lo = fmaf(t - magic, -4096.0f, v) + magic;
-    return static_cast<int>(__float_as_uint(t) * 4096u + __float_as_uint(lo) - (0x4B400000u * 4096u + 0x4B400000u));
-}
-
-__device__ __forceinline__ int acc_to_int(uint32_t bits, int k)
-{
-    return k % 8 < 3 ? __float2int_rn(__uint_as_float(bits)) : split_to_int(__uint_as_float(bits));
-}
-
 // 32 columns of the sums, from the hand-over's regions.
 __device__ __forceinline__ void load_sums(uint32_t addr, int regions, uint32_t stride, int (&v)[32])
 {

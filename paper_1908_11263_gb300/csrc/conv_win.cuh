@@ -31,7 +31,9 @@
 // the number of chunks from the filters themselves: the fewest contiguous tap
 // ranges for which max|staged x| * sum|w| over the range stays within 2^22 for
 // every output channel (the worst case over all filters is the planner's
-// nch_max, always valid).
+// nch_max, always valid).  INT-8 filters that need several such chunks run
+// without the pre-load where that needs fewer: sums up to 2^24 around 0, every
+// one an integer that fp32 holds exactly, converted to int32 by the epilogue.
 //
 // Filters in the kernel.  The loader first bulk-copies the packed filters and
 // the first windows' input rows; meanwhile the epilogue warps and the MMA warp
@@ -82,13 +84,14 @@ constexpr int kSmemLimit = 232448;    // 227 KB opt-in dynamic shared memory per
 // the MMAs per tile.
 struct Misc {
     uint32_t tmem;
-    uint32_t nch;  // accumulators per strip: exact chunks x K-split
+    uint32_t nch;  // accumulators (exact chunks) per strip
     uint32_t nslots;
     uint32_t slot_cols;
     uint32_t mask;
+    uint32_t mask24;  // the same for accumulators without the pre-load
     uint32_t nmma;  // MMAs per tile (entries of the issue table)
-    uint32_t kx;    // K-split: the k-steps of a tap alternate between kx accumulators
     uint32_t cst;   // TMEM column of the per-channel constants (lam2, then kappa), or ~0u: none
+    uint32_t fmode; // INT-8: accumulators start at 0 and hold integers up to 2^24 (no pre-load)
 };
 
 // Accumulator slots of `cols` columns each, and the 2 * NT columns of the
@@ -444,13 +447,12 @@ __device__ __forceinline__ void mma_nc(uint32_t d, uint64_t ad, uint64_t bd, uin
 }
 
 // One tile's MMAs with every offset known at compile time (one exact chunk,
-// KH x KW taps, KS k-steps per tap, S strips, k-step kk of a tap into the
-// strip's accumulator kk % KX): a descriptor is its template's low word plus
+// KH x KW taps, KS k-steps per tap, S strips): a descriptor is its template's low word plus
 // an offset (a start address field that cannot carry out of its 14 bits), so
-// each MMA costs an addition or two and the issue.  Consecutive MMAs go to
-// S * KX different accumulators: an MMA into the accumulator the previous one
-// wrote waits for it, so one chain runs at about half the tensor pipe's rate.
-template <int KH, int KW, int KS, int S, int NT, bool F8, int KX>
+// each MMA costs an addition or two and the issue.  (Consecutive MMAs into one
+// accumulator run at the full rate: 48.3 cycles at N = 64, one or two.)
+// START: the first MMA into an accumulator overwrites it (no pre-load).
+template <int KH, int KW, int KS, int S, int NT, bool F8, bool START>
 __device__ __forceinline__ void issue_fixed(uint32_t d0, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                             uint32_t idesc, int sp, uint32_t kstep_a)
 {
@@ -464,9 +466,12 @@ __device__ __forceinline__ void issue_fixed(uint32_t d0, uint32_t alo, uint32_t 
             for (int kk = 0; kk < KS; ++kk) {
                 const uint64_t bd = desc_of(blo + static_cast<uint32_t>(((i * KW + j) * 2 * KS + 2 * kk) * NT), bhi);
 #pragma unroll
-                for (int s = 0; s < S; ++s)
-                    mma_nc<F8>(d0 + (s * KX + kk % KX) * NT, desc_of(arow + j + kk * kstep_a + s * kCols, ahi), bd,
-                               idesc);
+                for (int s = 0; s < S; ++s) {
+                    const uint32_t d = d0 + s * NT;
+                    const uint64_t ad = desc_of(arow + j + kk * kstep_a + s * kCols, ahi);
+                    if (START && j == 0 && kk == 0) mma_f16_ss_warp_nc(d, ad, bd, idesc, static_cast<uint32_t>(i));
+                    else mma_nc<F8>(d, ad, bd, idesc);
+                }
             }
     }
 }
@@ -489,14 +494,14 @@ __device__ __forceinline__ void mma_role(const WinArgs &a, uint8_t *smem, uint64
     const uint32_t pre16 = smem_addr(smem + a.off_pre) >> 4;
     const uint64_t pre_a = smem_desc(0, 2048, 128) + pre16;
     const uint64_t pre_b = smem_desc(0, NT * 16, 128) + pre16 + 256;
-    const int nacc = a.s * nch;
-    const int kx = static_cast<int>(misc->kx);
+    const uint32_t keep = F8 || misc->fmode == 0 ? 1u : 0u;  // accumulators start at the pre-load
+    const int nacc = keep ? a.s * nch : 0;
     // the issue order (built by the filter preparation): one 8-byte entry per MMA,
-    // {A offset in 16-byte units | accumulator column << 16, B offset}
+    // {A offset in 16-byte units | first of its accumulator << 15 | accumulator column << 16, B offset}
     const uint2 *tab = reinterpret_cast<const uint2 *>(smem + a.off_mtab);
     const int nu = static_cast<int>(misc->nmma);
     // the common shapes with one exact chunk issue from unrolled code
-    const int fixed = nch != kx ? 0
+    const int fixed = nch != 1 ? 0
                       : (a.kh == 3 && a.kwf == 3 && a.ksteps == 2 && a.s == 2) ? 1
                       : (a.kh == 3 && a.kwf == 3 && a.ksteps == 1 && a.s == 2) ? 2
                       : (a.kh == 5 && a.kwf == 5 && a.ksteps == 2 && a.s == 2) ? 3
@@ -515,21 +520,29 @@ __device__ __forceinline__ void mma_role(const WinArgs &a, uint8_t *smem, uint64
         for (int b = 0; b < nacc; ++b) mma_f16_ss_warp_nc(d0 + b * NT, pre_a, pre_b, idesc, 0u);
         const uint32_t alo = static_cast<uint32_t>(abase), ahi = static_cast<uint32_t>(abase >> 32);
         const uint32_t blo = static_cast<uint32_t>(bbase), bhi = static_cast<uint32_t>(bbase >> 32);
-        switch (fixed * 2 + (kx == 2 ? 1 : 0)) {
-            case 2: issue_fixed<3, 3, 2, 2, NT, F8, 1>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 3: issue_fixed<3, 3, 2, 2, NT, F8, 2>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 4: issue_fixed<3, 3, 1, 2, NT, F8, 1>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 6: issue_fixed<5, 5, 2, 2, NT, F8, 1>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 7: issue_fixed<5, 5, 2, 2, NT, F8, 2>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 8: issue_fixed<5, 5, 2, 1, NT, F8, 1>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 9: issue_fixed<5, 5, 2, 1, NT, F8, 2>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 10: issue_fixed<3, 3, 4, 2, NT, F8, 1>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
-            case 11: issue_fixed<3, 3, 4, 2, NT, F8, 2>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break;
+        // (no staging but INT-8's goes without the pre-load)
+        constexpr bool kStart = !F8;
+        switch (fixed * 2 + (keep ? 0 : 1)) {
+#define QNN_ISSUE(KH, KW, KS, S, ST) \
+    issue_fixed<KH, KW, KS, S, NT, F8, ST>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break
+            case 2: QNN_ISSUE(3, 3, 2, 2, false);
+            case 4: QNN_ISSUE(3, 3, 1, 2, false);
+            case 6: QNN_ISSUE(5, 5, 2, 2, false);
+            case 8: QNN_ISSUE(5, 5, 2, 1, false);
+            case 10: QNN_ISSUE(3, 3, 4, 2, false);
+            // without the pre-load: long filters only
+            case 7: QNN_ISSUE(5, 5, 2, 2, kStart);
+            case 9: QNN_ISSUE(5, 5, 2, 1, kStart);
+            case 11: QNN_ISSUE(3, 3, 4, 2, kStart);
+#undef QNN_ISSUE
             default:
 #pragma unroll 4
                 for (int u = 0; u < nu; ++u) {
                     const uint2 e = tab[u];
-                    mma_nc<F8>(d0 + (e.x >> 16), abase + (e.x & 0xFFFFu), bbase + e.y, idesc);
+                    if (F8) mma_nc<F8>(d0 + (e.x >> 16), abase + (e.x & 0x7FFFu), bbase + e.y, idesc);
+                    else
+                        mma_f16_ss_warp_nc(d0 + (e.x >> 16), abase + (e.x & 0x7FFFu), bbase + e.y, idesc,
+                                           keep | (~e.x >> 15 & 1u));
                 }
         }
         mma_commit_warp(&acc_full[slot]);
@@ -618,7 +631,7 @@ __device__ __forceinline__ void prepare_filters(const WinArgs &a, uint8_t *smem,
     int *tapabs = reinterpret_cast<int *>(smem + a.off_tap);    // [taps][NT]
     int *sums = tapabs + a.taps * NT;                           // [2][NT]: positive part, negative part
     for (int i = et; i < 2 * NT; i += kPrepThreads) sums[i] = 0;
-    if (et == 0) misc->mask = ~0u;
+    if (et == 0) misc->mask = misc->mask24 = ~0u;
     prep_sync();
     // item i: channel n = i % NT, tap i / NT; thread et takes items et, et + kPrepThreads, ...
     // K-chunks holding filter values, and packed bytes of one tap of one filter (a kernel
@@ -698,29 +711,35 @@ __device__ __forceinline__ void prepare_filters(const WinArgs &a, uint8_t *smem,
     // nch_max) holds by the planner's worst-case bound whatever the filters.
     const int c_force = max(a.nch_min, a.nch_max);
     if (et < NT) {
-        uint32_t okmask = 0;
+        uint32_t okmask = 0, okmask24 = 0;
         for (int c = a.nch_min; c <= c_force; ++c) {
             const int ct = (a.taps + c - 1) / c;
             if ((c - 1) * ct >= a.taps) continue;  // an empty chunk: not a c-chunk split
-            bool good = true;
-            for (int j = 0; j < c && good; ++j) {
+            long long most = 0;
+            for (int j = 0; j < c; ++j) {
                 long long b = 0;
                 for (int tap = j * ct; tap < min(a.taps, (j + 1) * ct); ++tap) b += tapabs[tap * NT + et];
-                good = b * kMaxX <= (1ll << 22);
+                most = max(most, b * kMaxX);
             }
-            if (good) okmask |= 1u << c;
+            if (most <= (1ll << 22)) okmask |= 1u << c;
+            if (most <= (1ll << 24)) okmask24 |= 1u << c;
         }
         okmask |= 1u << c_force;
+        okmask24 |= 1u << c_force;
         atomicAnd(&misc->mask, okmask);
+        atomicAnd(&misc->mask24, okmask24);
     }
     prep_sync();
-    const int nch = __ffs(static_cast<int>(misc->mask)) - 1;
-    // K-split: a tile with a single accumulator (one strip, one chunk) and an
-    // even k-step count alternates the k-steps of a tap between two
-    // accumulators (each sums a subset of the chunk's products, so each is
-    // exact where the chunk is), so that consecutive MMAs do not wait on each
-    // other; the epilogue adds all nch * kx accumulators of a strip
-    const int kx = (a.s * nch == 1 && a.ksteps % 2 == 0 && 2 * NT <= 256) ? 2 : 1;
+    // INT-8 filters too large for one chunk around the pre-load start their
+    // accumulators at 0 instead, where fp32 holds integers up to 2^24: the
+    // accumulators then need a conversion in the epilogue (acc_to_int), and
+    // halving their number is worth more: one chunk issues from unrolled code
+    // (the table's entries took about 85 cycles per MMA, 48 unrolled), leaves
+    // TMEM for the constants and is read once.  56 x 56 x 64 -> 64 3 x 3, batch
+    // 256: 98.0 -> 74.5 us; CIFAR-shaped network, batch 1,024: 110 -> 99.7 us.
+    const int nch22 = __ffs(static_cast<int>(misc->mask)) - 1, nch24 = __ffs(static_cast<int>(misc->mask24)) - 1;
+    const bool fmode = BITS == 8 && nch24 < nch22 && nch24 <= 2;
+    const int nch = fmode ? nch24 : nch22;
     // The MMA issue order, one 8-byte entry per MMA: {A offset (16-byte units
     // within a stage) | accumulator column << 16, B offset}.  The accumulators
     // (chunk c, strip s) are independent and consecutive MMAs go to different
@@ -740,17 +759,18 @@ __device__ __forceinline__ void prepare_filters(const WinArgs &a, uint8_t *smem,
             const int tap = c * ct + jt, ti = tap / a.kwf, tj = tap - ti * a.kwf;
             for (int s = 0; s < a.s; ++s, ++u)
                 tab[u] = make_uint2((static_cast<uint32_t>(ti * a.sp + tj) + kk * kstep_a + s * kCols) |
-                                        (static_cast<uint32_t>((s * nch + c) * kx + kk % kx) * NT << 16),
+                                        (jt == 0 && kk == 0 ? 0x8000u : 0u) |
+                                        (static_cast<uint32_t>(s * nch + c) * NT << 16),
                                     static_cast<uint32_t>(tap * a.groups) * NT + kk * kstep_b);
         }
     }
     if (et == 0) {
-        const uint32_t cols = static_cast<uint32_t>(a.s * nch * kx * NT);
-        misc->nch = static_cast<uint32_t>(nch * kx);
-        misc->kx = static_cast<uint32_t>(kx);
-        // the tap area's spare row carries both into a prepared image
-        tapabs[(a.taps + 2) * NT] = nch * kx;
-        tapabs[(a.taps + 2) * NT + 1] = kx;
+        const uint32_t cols = static_cast<uint32_t>(a.s * nch * NT);
+        misc->nch = static_cast<uint32_t>(nch);
+        // the tap area's spare row carries these into a prepared image
+        tapabs[(a.taps + 2) * NT] = nch;
+        tapabs[(a.taps + 2) * NT + 1] = fmode ? 1 : 0;
+        misc->fmode = fmode ? 1u : 0u;
         slot_layout<NT>(misc, cols);
         misc->nmma = static_cast<uint32_t>(a.s * a.taps * a.ksteps);
     }
@@ -775,7 +795,7 @@ __device__ __forceinline__ void prepare_records(const WinArgs &a, uint8_t *smem,
 {
     const int et = threadIdx.x - kEpiWarp0 * 32;
     const int *sums = reinterpret_cast<const int *>(smem + a.off_tap) + a.taps * NT;
-    const int nch = static_cast<int>(misc->nch);
+    const int nch = misc->fmode ? 0 : static_cast<int>(misc->nch);  // pre-loads to remove
     int4 *rec0 = reinterpret_cast<int4 *>(smem + a.off_rec);
     int4 *rec1 = rec0 + NT;
     if (et < NT) {
@@ -783,15 +803,34 @@ __device__ __forceinline__ void prepare_records(const WinArgs &a, uint8_t *smem,
         const long long off = BITS == 8 ? -128 : 0;  // staged activation = x + off
         const int s_w = sums[o] + sums[NT + o];
         int4 r0 = make_int4(0, 0, 0, kModeDirect), r1 = make_int4(0, 0, 0, 0);
-        if (a.thr) {
-            // staircase: the epilogue compares acc = s + beta with the thresholds
-            const uint32_t beta = 0u - static_cast<uint32_t>(off * s_w) - static_cast<uint32_t>(nch) * kMagic;
-            int32_t *ts = reinterpret_cast<int32_t *>(smem + a.off_thr) + o * kThrStride;
-            for (int k = 0; k < kThrStride; ++k)
-                ts[k] = (o < a.m && k < (1 << BITS) - 1) ? a.thr[static_cast<long long>(o) * ((1 << BITS) - 1) + k]
-                                                        : INT32_MAX;
-            r0 = make_int4(static_cast<int>(a.off_thr) + o * 4 * kThrStride, 0, 0, kModeThreshold);
-            r1 = make_int4(static_cast<int32_t>(beta), 0, 0, 0);
+        if (BITS != 8 && a.thr) {
+            // Staircase: the number of thresholds that do not exceed acc does not
+            // depend on their order, so they are sorted, and brought to the raw sums:
+            // acc = s - nch * kMagic, and s is within 2^26 of a constant that is further
+            // than that from the ends of int32, so threshold + nch * kMagic, cut to
+            // int32, compares with s as the threshold with acc.
+            const long long shift = static_cast<int32_t>(static_cast<uint32_t>(nch) * kMagic);
+            constexpr int kCount = BITS == 8 ? 0 : (1 << BITS) - 1;  // (no staircase at INT-8)
+            int32_t t[kThrStride];
+#pragma unroll
+            for (int k = 0; k < kThrStride; ++k) {
+                long long v = INT32_MAX;
+                if (o < a.m && k < kCount) v = a.thr[static_cast<long long>(o) * kCount + k] + shift;
+                t[k] = static_cast<int32_t>(v < INT32_MIN ? INT32_MIN : v > INT32_MAX ? INT32_MAX : v);
+            }
+            // odd-even transposition (BITS 4: 15 values, BITS 2: 3)
+#pragma unroll
+            for (int round = 0; round < kCount; ++round)
+#pragma unroll
+                for (int k = round & 1; k + 1 < kCount; k += 2) {
+                    const int32_t lo = min(t[k], t[k + 1]), hi = max(t[k], t[k + 1]);
+                    t[k] = lo;
+                    t[k + 1] = hi;
+                }
+            int4 *ts = reinterpret_cast<int4 *>(smem + a.off_thr) + o * (kThrStride / 4);
+#pragma unroll
+            for (int k = 0; k < kThrStride / 4; ++k) ts[k] = make_int4(t[4 * k], t[4 * k + 1], t[4 * k + 2], t[4 * k + 3]);
+            r0 = BITS == 4 ? make_int4(t[3], t[7], t[11], kModeThreshold) : make_int4(t[0], t[1], t[2], kModeThreshold);
         } else if (o < a.m) {
             const int32_t b = a.bias ? a.bias[o] : 0;
             const uint32_t beta = static_cast<uint32_t>(b) - static_cast<uint32_t>(off * s_w) -
@@ -845,7 +884,7 @@ __device__ __forceinline__ void image_ready(const WinArgs &a, uint8_t *smem, Mis
         const int *spare = reinterpret_cast<const int *>(smem + a.off_tap) + (a.taps + 2) * NT;
         const uint32_t nacc = static_cast<uint32_t>(spare[0]), cols = static_cast<uint32_t>(a.s) * nacc * NT;
         misc->nch = nacc;
-        misc->kx = static_cast<uint32_t>(spare[1]);
+        misc->fmode = static_cast<uint32_t>(spare[1]);
         slot_layout<NT>(misc, cols);
         misc->nmma = static_cast<uint32_t>(a.s * a.taps * a.ksteps);
     }
@@ -882,10 +921,11 @@ __device__ __forceinline__ void tmem_load(uint32_t addr, uint32_t (&v)[EB])
     }
 }
 
-// More than two chunks (long filters with large weights): one wait per chunk.
+// Any number of chunks, one wait each (fmode: accumulators without the
+// pre-load, converted to int32).
 template <int EB>
-__device__ __forceinline__ void drain_many(uint32_t a0, uint32_t a1, bool two, int nch, uint32_t stride, uint32_t (&v0)[EB],
-                                        uint32_t (&v1)[EB])
+__device__ __forceinline__ void drain_many(uint32_t a0, uint32_t a1, bool two, int nch, uint32_t stride, bool fmode,
+                                           uint32_t (&v0)[EB], uint32_t (&v1)[EB])
 {
 #pragma unroll
     for (int k = 0; k < EB; ++k) v0[k] = v1[k] = 0;
@@ -897,34 +937,9 @@ __device__ __forceinline__ void drain_many(uint32_t a0, uint32_t a1, bool two, i
         tmem_wait_ld();
 #pragma unroll
         for (int k = 0; k < EB; ++k) {
-            v0[k] += t0[k];
-            v1[k] += t1[k];
+            v0[k] += fmode ? static_cast<uint32_t>(acc_to_int(t0[k], 0)) : t0[k];
+            v1[k] += fmode ? static_cast<uint32_t>(acc_to_int(t1[k], 0)) : t1[k];
         }
-    }
-}
-
-template <int EB>
-__device__ __forceinline__ void drain_block(uint32_t a0, uint32_t a1, bool two, int nch, uint32_t stride,
-                                            uint32_t (&v0)[EB], uint32_t (&v1)[EB])
-{
-    if (nch <= 2) {
-        uint32_t t0[EB], t1[EB];
-        tmem_load<EB>(a0, v0);
-        if (nch == 2) tmem_load<EB>(a0 + stride, t0);
-        if (two) {
-            tmem_load<EB>(a1, v1);
-            if (nch == 2) tmem_load<EB>(a1 + stride, t1);
-        }
-        tmem_wait_ld();
-        if (nch == 2) {
-#pragma unroll
-            for (int k = 0; k < EB; ++k) {
-                v0[k] += t0[k];
-                v1[k] += t1[k];  // unused when !two
-            }
-        }
-    } else {
-        drain_many<EB>(a0, a1, two, nch, stride, v0, v1);
     }
 }
 
@@ -981,60 +996,89 @@ __device__ __forceinline__ void store_words(uint32_t (&pk)[(HB * BITS + 31) / 32
     if (store) store_packed<BITS, HB>(pk, valid, dst);
 }
 
-// Whether channel m's compression is in the direct form (flags per 16 channels).
-__device__ __forceinline__ bool l_direct(const uint8_t *gdirect, int m) { return gdirect[m >> 4] != 0; }
+// How a warp's channels are compressed.  Each kind has its own copy of the
+// block loop, so that the registers of the others do not weigh on it (with the
+// kinds told apart inside one loop the INT-2 layer at batch 2,048 spilled and
+// took 35.6 us instead of 30.9).
+enum EpiKind {
+    kEpiDirect = 0,  // direct form, one shift; constants from TMEM with the accumulators
+    kEpiShifts = 1,  // the same with a shift per channel, kept above kappa
+    kEpiShfl = 2,    // direct form, no room in TMEM: constants broadcast from registers
+    kEpiThr = 3,     // staircase
+    kEpiRec = 4      // any form, any number of accumulators; records from shared memory
+};
 
 // One tile's epilogue state for a warp: its TMEM columns, channels, output
-// pixels and whether the direct form with one shift covers all its channels.
-template <int NT>
+// pixels.
 struct EpiTile {
     uint32_t base, strip1;
-    bool two;
+    bool two, fmode;
     int nch, col0, lane;
-    bool direct_all, one_shift;
-    uint32_t shift;
+    uint32_t shift;    // kEpiDirect
     const int4 *rec0, *rec1;
+    const int4 *thr;   // kEpiThr: each channel's sorted thresholds, 16 apart
     uint8_t *dst[2];
     bool store[2];
     uint64_t *acc_empty;
-    bool tmem_cst;     // lam2 and kappa of the block's channels come from TMEM with the accumulators
     uint32_t cst_addr; // TMEM address of lam2 of channel col0 in this warp's lanes (kappa NT columns on)
 };
 
-// The tile's columns in blocks of HB: the loads of a block (NCH accumulators
-// per strip, 0 = any count, one wait per accumulator), the slot released
+// Staircase of Eq. 4 on a raw sum: how many of the channel's sorted thresholds
+// do not exceed it.  INT-4: the quarter by three pivots (piv, the same for all
+// lanes), then the three thresholds within it, one 16-byte load; 15 loads and
+// compares per value, with a call, took the INT-4 benchmark layer at batch 512
+// to 70 us, this 20.
+template <int BITS>
+__device__ __forceinline__ int staircase(int32_t s, int4 piv, const int4 *tau)
+{
+    const int g = (piv.x <= s ? 1 : 0) + (piv.y <= s ? 1 : 0) + (piv.z <= s ? 1 : 0);
+    if (BITS == 2) return g;
+    const int4 t = tau[g];
+    return 4 * g + (t.x <= s ? 1 : 0) + (t.y <= s ? 1 : 0) + (t.z <= s ? 1 : 0);
+}
+
+// The tile's columns in blocks of HB: the loads of a block (one accumulator
+// per strip; kEpiRec: any count, one wait per accumulator), the slot released
 // after the last block's loads, then compression, packing and stores (HB
-// values of a pixel are HB * Q / 8 contiguous bytes).
-template <int BITS, int NT, bool POOL, int HB, int NCH>
-__device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile<NT> &e, const uint32_t (&my_lam2)[2],
-                                         const uint32_t (&my_kap)[2], const uint32_t (&my_sh)[2])
+// values of a pixel are HB * Q / 8 contiguous bytes).  FM: accumulators without
+// the pre-load.
+template <int BITS, int NT, bool POOL, int HB, int KIND, bool FM>
+__device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile &e)
 {
     constexpr int CW = NT / 2;
+    constexpr bool kCst = KIND == kEpiDirect || KIND == kEpiShifts;
+    // kEpiShfl: the constants of channel col0 + c sit in lane c % 32 of set c / 32
+    uint32_t my_lam2[2], my_kap[2], my_sh[2];
+    if constexpr (KIND == kEpiShfl) {
+        constexpr int LW = CW < 32 ? CW : 32;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int4 rec = e.rec0[e.col0 + (r * 32 < CW ? r * 32 : 0) + e.lane % LW];
+            my_lam2[r] = static_cast<uint32_t>(rec.x);
+            my_kap[r] = static_cast<uint32_t>(rec.y);
+            my_sh[r] = static_cast<uint32_t>(rec.z);
+        }
+    }
 #pragma unroll 1
     for (int k0 = 0; k0 < CW; k0 += HB) {
-        uint32_t v0[HB], v1[HB], cl[HB], ck[HB];  // accumulators; lam2 and kappa when tmem_cst
-        if constexpr (NCH == 0) {
-            drain_many<HB>(e.base + k0, e.base + e.strip1 + k0, e.two, e.nch, NT, v0, v1);
+        uint32_t v0[HB], v1[HB], cl[HB], ck[HB];  // accumulators; lam2 and kappa
+        if constexpr (KIND == kEpiRec) {
+            drain_many<HB>(e.base + k0, e.base + e.strip1 + k0, e.two, e.nch, NT, e.fmode, v0, v1);
         } else {
-            uint32_t t0[NCH == 2 ? HB : 1], t1[NCH == 2 ? HB : 1];
-            if (e.tmem_cst) {
+            if constexpr (kCst) {
                 tmem_load<HB>(e.cst_addr + k0, cl);
                 tmem_load<HB>(e.cst_addr + NT + k0, ck);
             }
             tmem_load<HB>(e.base + k0, v0);
-            if constexpr (NCH == 2) tmem_load<HB>(e.base + k0 + NT, t0);
-            if (e.two) {
-                tmem_load<HB>(e.base + e.strip1 + k0, v1);
-                if constexpr (NCH == 2) tmem_load<HB>(e.base + e.strip1 + k0 + NT, t1);
-            }
+            if (e.two) tmem_load<HB>(e.base + e.strip1 + k0, v1);
             tmem_wait_ld();
 #pragma unroll
             for (int k = 0; k < HB; ++k) {
-                asm volatile("" : "+r"(v0[k]), "+r"(v1[k]), "+r"(cl[k]), "+r"(ck[k]));  // uses stay after the wait
-                if constexpr (NCH == 2) {
-                    asm volatile("" : "+r"(t0[k]), "+r"(t1[k]));
-                    v0[k] += t0[k];
-                    v1[k] += t1[k];  // unused when !two
+                asm volatile("" : "+r"(v0[k]), "+r"(v1[k]));  // uses stay after the wait
+                if constexpr (kCst) asm volatile("" : "+r"(cl[k]), "+r"(ck[k]));
+                if constexpr (FM) {
+                    v0[k] = static_cast<uint32_t>(acc_to_int(v0[k], k));
+                    v1[k] = static_cast<uint32_t>(acc_to_int(v1[k], k + 4));
                 }
             }
         }
@@ -1053,32 +1097,43 @@ __device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile<NT> &e,
 #pragma unroll
         for (int g0 = 0; g0 < HB; g0 += kG) {
             int y0[kG], y1[kG];
-            if (NCH != 0 && e.tmem_cst) {
-                // direct form, one shift: the constants arrived with the accumulators
 #pragma unroll
-                for (int k = 0; k < kG; ++k) {
+            for (int k = 0; k < kG; ++k) {
+                // direct channels: ((s * kappa + lam2) mod 2^32) >> shift is exact (see the records)
+                if constexpr (KIND == kEpiDirect) {
                     y0[k] = static_cast<int32_t>(v0[g0 + k] * ck[g0 + k] + cl[g0 + k]) >> e.shift;
                     y1[k] = static_cast<int32_t>(v1[g0 + k] * ck[g0 + k] + cl[g0 + k]) >> e.shift;
-                }
-            } else if (e.direct_all) {
-                // direct channels: ((s * kappa + lam2) mod 2^32) >> shift is exact (see the records);
-                // the constants of channel col0 + k0 + k sit in lane (k0 + k) % 32 of set (k0 + k) / 32
-#pragma unroll
-                for (int k = 0; k < kG; ++k) {
+                } else if constexpr (KIND == kEpiShifts) {
+                    const uint32_t kap = static_cast<uint32_t>(static_cast<int32_t>(ck[g0 + k] << 16) >> 16);
+                    const uint32_t sh = ck[g0 + k] >> 16;
+                    y0[k] = static_cast<int32_t>(v0[g0 + k] * kap + cl[g0 + k]) >> sh;
+                    y1[k] = static_cast<int32_t>(v1[g0 + k] * kap + cl[g0 + k]) >> sh;
+                } else if constexpr (KIND == kEpiShfl) {
                     const int c = k0 + g0 + k, set = c >= 32 ? 1 : 0;
                     const uint32_t lam2 = __shfl_sync(0xffffffffu, set ? my_lam2[1] : my_lam2[0], c & 31);
                     const uint32_t kap = __shfl_sync(0xffffffffu, set ? my_kap[1] : my_kap[0], c & 31);
-                    const uint32_t sh =
-                        e.one_shift ? e.shift : __shfl_sync(0xffffffffu, set ? my_sh[1] : my_sh[0], c & 31);
+                    const uint32_t sh = __shfl_sync(0xffffffffu, set ? my_sh[1] : my_sh[0], c & 31);
                     y0[k] = static_cast<int32_t>(v0[g0 + k] * kap + lam2) >> sh;
                     y1[k] = static_cast<int32_t>(v1[g0 + k] * kap + lam2) >> sh;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < kG; ++k) {
+                } else if constexpr (KIND == kEpiThr) {
+                    const int4 piv = e.rec0[m0 + g0 + k];
+                    const int4 *tau = e.thr + (m0 + g0 + k) * (kThrStride / 4);
+                    y0[k] = staircase<BITS>(static_cast<int32_t>(v0[g0 + k]), piv, tau);
+                    y1[k] = staircase<BITS>(static_cast<int32_t>(v1[g0 + k]), piv, tau);
+                } else {
                     const int4 r0 = e.rec0[m0 + g0 + k], r1 = e.rec1[m0 + g0 + k];
-                    y0[k] = static_cast<int>(compress_slow(v0[g0 + k], r0, r1, (1u << BITS) - 1u));
-                    y1[k] = e.two ? static_cast<int>(compress_slow(v1[g0 + k], r0, r1, (1u << BITS) - 1u)) : 0;
+                    if (BITS != 8 && e.thr) {
+                        y0[k] = staircase<BITS>(static_cast<int32_t>(v0[g0 + k]), r0,
+                                                e.thr + (m0 + g0 + k) * (kThrStride / 4));
+                        y1[k] = staircase<BITS>(static_cast<int32_t>(v1[g0 + k]), r0,
+                                                e.thr + (m0 + g0 + k) * (kThrStride / 4));
+                    } else if (r0.w == kModeDirect) {
+                        y0[k] = static_cast<int32_t>(v0[g0 + k] * r0.y + r0.x) >> r0.z;
+                        y1[k] = static_cast<int32_t>(v1[g0 + k] * r0.y + r0.x) >> r0.z;
+                    } else {
+                        y0[k] = static_cast<int>(compress_slow(v0[g0 + k], r0, r1, (1u << BITS) - 1u));
+                        y1[k] = e.two ? static_cast<int>(compress_slow(v1[g0 + k], r0, r1, (1u << BITS) - 1u)) : 0;
+                    }
                 }
             }
             pack_values<BITS, kG>(y0, *reinterpret_cast<uint32_t(*)[kGW]>(pk0 + g0 / kG * kGW));
@@ -1107,24 +1162,16 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
     const uint8_t *gdirect = reinterpret_cast<const uint8_t *>(rec1 + NT);
     const int out_row_bytes = a.m * BITS / 8;
     const bool two = a.s == 2;
-    // This warp's channels are fixed: lane l keeps channel col0 + l's direct-form
-    // constants in registers and broadcasts them with shuffles, so the inner loop
-    // touches no shared memory (the tensor cores keep it busy with operand reads).
-    constexpr int LW = CW < 32 ? CW : 32;  // channels per register set
-    uint32_t my_lam2[2], my_kap[2], my_sh[2];
-    bool direct_all = true;
+    // whether the direct form covers this warp's channels (flags per 16 channels), and with one shift
+    constexpr int LW = CW < 32 ? CW : 32;
+    const uint32_t shift = static_cast<uint32_t>(rec0[col0].z);
+    bool direct_all = true, one_shift = true;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int m = col0 + (r * 32 < CW ? r * 32 : 0) + lane % LW;
-        const int4 rec = rec0[m];
-        my_lam2[r] = static_cast<uint32_t>(rec.x);
-        my_kap[r] = static_cast<uint32_t>(rec.y);
-        my_sh[r] = static_cast<uint32_t>(rec.z);
-        direct_all = __all_sync(0xffffffffu, l_direct(gdirect, m)) && direct_all;
+    for (int r = 0; r < (CW + 31) / 32; ++r) {
+        const int m = col0 + r * 32 + lane % LW;
+        direct_all = __all_sync(0xffffffffu, gdirect[m >> 4] != 0) && direct_all;
+        one_shift = __all_sync(0xffffffffu, static_cast<uint32_t>(rec0[m].z) == shift) && one_shift;
     }
-    // one shift for all of this warp's channels: the common case, one shuffle less per value
-    const uint32_t shift = __shfl_sync(0xffffffffu, my_sh[0], 0);
-    const bool one_shift = __all_sync(0xffffffffu, my_sh[0] == shift && my_sh[1] == shift);
     const uint32_t strip1 = static_cast<uint32_t>(nch) * NT;  // columns from strip 0's buffers to strip 1's
     int *const status = a.status;
     // The direct-form constants of this warp's channels, one row per lane of its
@@ -1132,7 +1179,7 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
     // instead of broadcasting them lane to lane (shuffles queue behind the
     // tensor cores' shared-memory reads).
     const uint32_t cst = misc->cst;
-    const bool tmem_cst = cst != ~0u && direct_all && one_shift;
+    const bool tmem_cst = cst != ~0u && direct_all;
     const uint32_t cst_addr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + cst + col0;
     if (tmem_cst) {
 #pragma unroll 1
@@ -1142,13 +1189,20 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
             for (int k = 0; k < 16; ++k) {
                 const int4 r = rec0[col0 + j + k];
                 l[k] = static_cast<uint32_t>(r.x);
-                kp[k] = static_cast<uint32_t>(r.y);
+                kp[k] = one_shift ? static_cast<uint32_t>(r.y)
+                                  : (static_cast<uint32_t>(r.y) & 0xFFFFu) | static_cast<uint32_t>(r.z) << 16;
             }
             tmem_st16(cst_addr + j, l);
             tmem_st16(cst_addr + NT + j, kp);
         }
         tmem_wait_st();
     }
+
+    const int4 *thr = a.thr ? reinterpret_cast<const int4 *>(smem + a.off_thr) : nullptr;
+    const bool fmode = BITS == 8 && misc->fmode != 0;
+    // kind * 2 + 1 without the pre-load; several accumulators per strip run from the records
+    const int kind = thr ? kEpiThr : !direct_all ? kEpiRec : tmem_cst ? (one_shift ? kEpiDirect : kEpiShifts) : kEpiShfl;
+    const int variant = nch > 1 ? 2 * kEpiRec : 2 * kind + (fmode ? 1 : 0);
 
     const int oyr = row >> 3, oxr = row & 7;
     for (int i = 0, t = blockIdx.x; t < a.total_tiles; ++i, t += gridDim.x) {
@@ -1174,16 +1228,23 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
             }
             store[s] = store[s] && (s == 0 || two);
         }
-        const uint32_t base = lane_addr + slot * slot_cols;
-        const EpiTile<NT> et{base,     strip1,  two,   nch,  col0,     lane,
-                             direct_all, one_shift, shift, rec0, rec1,  {dst[0], dst[1]},
-                             {store[0], store[1]}, &acc_empty[slot], tmem_cst, cst_addr};
-        // every load of a block of 8 columns (both strips' accumulators and, with
-        // tmem_cst, the constants) goes out before one wait; more than two
-        // accumulators per strip: one wait per accumulator
-        if (nch == 1) epi_tile<BITS, NT, POOL, (CW < 8 ? CW : 8), 1>(a, et, my_lam2, my_kap, my_sh);
-        else if (nch == 2) epi_tile<BITS, NT, POOL, (CW < 8 ? CW : 8), 2>(a, et, my_lam2, my_kap, my_sh);
-        else epi_tile<BITS, NT, POOL, (CW < 8 ? CW : 8), 0>(a, et, my_lam2, my_kap, my_sh);
+        const EpiTile et{lane_addr + slot * slot_cols, strip1, two, fmode, nch, col0, lane, shift, rec0, rec1, thr,
+                         {dst[0], dst[1]}, {store[0], store[1]}, &acc_empty[slot], cst_addr};
+        // every load of a block of 8 columns (both strips' accumulators and the
+        // constants) goes out before one wait
+        constexpr int HB = CW < 8 ? CW : 8;
+#define QNN_EPI(KIND, FM) epi_tile<BITS, NT, POOL, HB, KIND, FM>(a, et); break
+        switch (variant) {
+            case 2 * kEpiDirect: QNN_EPI(kEpiDirect, false);
+            case 2 * kEpiShifts: QNN_EPI(kEpiShifts, false);
+            case 2 * kEpiShfl: QNN_EPI(kEpiShfl, false);
+            case 2 * kEpiThr: if constexpr (BITS != 8) { QNN_EPI(kEpiThr, false); }
+            case 2 * kEpiDirect + 1: if constexpr (BITS == 8) { QNN_EPI(kEpiDirect, true); }
+            case 2 * kEpiShifts + 1: if constexpr (BITS == 8) { QNN_EPI(kEpiShifts, true); }
+            case 2 * kEpiShfl + 1: if constexpr (BITS == 8) { QNN_EPI(kEpiShfl, true); }
+            default: epi_tile<BITS, NT, POOL, HB, kEpiRec, false>(a, et);
+        }
+#undef QNN_EPI
     }
 }
 
