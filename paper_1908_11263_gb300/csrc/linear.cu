@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace qnn {
@@ -70,6 +71,8 @@ constexpr int kSmemRowsMax = 200 * 1024;  // weight bytes kept in shared memory
 __global__ void __launch_bounds__(256) linear_smem_kernel(int n, int k, int m, const uint8_t *x, const int8_t *w,
                                                           const int32_t *bias, int32_t *y)
 {
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ uint4 wsh[];  // [m][k/16]
     const int kv = k / 16;
     const uint4 *wg = reinterpret_cast<const uint4 *>(w);
@@ -133,8 +136,7 @@ cudaError_t launch_linear(int n, int k, int m, const uint8_t *x, const int8_t *w
         }
         // enough warps to cover the rows, at most a few blocks per SM
         const int blocks = static_cast<int>(std::min<long long>((n + 7) / 8, 4ll * device_sm_count()));
-        linear_smem_kernel<<<blocks, 256, wbytes, st>>>(n, k, m, x, w, bias, y);
-        return cudaGetLastError();
+        return launch_pdl(linear_smem_kernel, static_cast<unsigned>(blocks), 256, wbytes, st, n, k, m, x, w, bias, y);
     }
     const unsigned grid = static_cast<unsigned>((n + 7) / 8);
     const bool vec = k % 4 == 0 && (reinterpret_cast<uintptr_t>(x) % 4) == 0 && (reinterpret_cast<uintptr_t>(w) % 4) == 0;

@@ -4,6 +4,7 @@
 // layout).  No padding, floor output size.
 #include <cstdint>
 
+#include "conv_common.cuh"
 #include "device.cuh"
 #include "internal.h"
 
@@ -11,29 +12,41 @@ namespace qnn {
 namespace {
 
 // One thread produces one 16-byte vector of an output pixel (pixels whose bytes
-// are whole 16-byte vectors).
-template <int BITS>
-__global__ void __launch_bounds__(256) maxpool_vec_kernel(int n, int h, int w, int vec_per_pix, int k, int s, int oh,
-                                                          int ow, const uint4 *x, uint4 *y)
+// are whole 16-byte vectors; at most 2^31 of them).  Bound by HBM; the index
+// takes three multiplications (64-bit divisions by run-time sizes took longer
+// than the loads), and the four loads of the 2 x 2 window go out together.
+// INT-2 2048 x 16 x 16 x 64: 2.6 us (6.9).
+template <int BITS, bool TWO>
+__global__ void __launch_bounds__(256) maxpool_vec_kernel(unsigned total, int h, int w, int vec_per_pix, int k, int s,
+                                                          FastDiv fd_vec, FastDiv fd_ow, FastDiv fd_oh, const uint4 *x,
+                                                          uint4 *y)
 {
-    const long long total = static_cast<long long>(n) * oh * ow * vec_per_pix;
-    const long long gid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    pdl_trigger();
+    pdl_wait();
+    const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= total) return;
-    const int v = static_cast<int>(gid % vec_per_pix);
-    const long long pix = gid / vec_per_pix;
-    const int ox = static_cast<int>(pix % ow);
-    const int oy = static_cast<int>((pix / ow) % oh);
-    const int b = static_cast<int>(pix / (static_cast<long long>(ow) * oh));
+    const int pix = fdiv(static_cast<int>(gid), fd_vec), v = static_cast<int>(gid) - pix * vec_per_pix;
+    const int row = fdiv(pix, fd_ow), ox = pix - row * static_cast<int>(fd_ow.d);
+    const int b = fdiv(row, fd_oh), oy = row - b * static_cast<int>(fd_oh.d);
+    const uint4 *src = x + ((static_cast<long long>(b) * h + oy * s) * w + ox * s) * vec_per_pix + v;
     uint4 best = make_uint4(0, 0, 0, 0);
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) {
-            const long long src = ((static_cast<long long>(b) * h + oy * s + i) * w + ox * s + j) * vec_per_pix + v;
-            const uint4 t = __ldg(x + src);
-            best.x = max_fields<BITS>(best.x, t.x);
-            best.y = max_fields<BITS>(best.y, t.y);
-            best.z = max_fields<BITS>(best.z, t.z);
-            best.w = max_fields<BITS>(best.w, t.w);
-        }
+    auto take = [&](const uint4 &t) {
+        best.x = max_fields<BITS>(best.x, t.x);
+        best.y = max_fields<BITS>(best.y, t.y);
+        best.z = max_fields<BITS>(best.z, t.z);
+        best.w = max_fields<BITS>(best.w, t.w);
+    };
+    if (TWO) {
+        const uint4 *low = src + static_cast<long long>(w) * vec_per_pix;
+        const uint4 t0 = __ldg(src), t1 = __ldg(src + vec_per_pix), t2 = __ldg(low), t3 = __ldg(low + vec_per_pix);
+        take(t0);
+        take(t1);
+        take(t2);
+        take(t3);
+    } else {
+        for (int i = 0; i < k; ++i)
+            for (int j = 0; j < k; ++j) take(__ldg(src + (static_cast<long long>(i) * w + j) * vec_per_pix));
+    }
     y[gid] = best;
 }
 
@@ -79,15 +92,21 @@ cudaError_t launch_maxpool(int n, int h, int w, int c, int k, int s, int bits, c
     const int bytes_per_pix = c * bits / 8;
     const bool vec = bytes_per_pix % 16 == 0 && (reinterpret_cast<uintptr_t>(x) % 16) == 0 &&
                      (reinterpret_cast<uintptr_t>(y) % 16) == 0;
-    if (vec) {
+    if (vec && pix * (bytes_per_pix / 16) < (1ll << 31)) {
         const int vpp = bytes_per_pix / 16;
-        const long long total = pix * vpp;
-        const unsigned grid = static_cast<unsigned>((total + 255) / 256);
+        const unsigned total = static_cast<unsigned>(pix * vpp), grid = (total + 255u) / 256u;
+        const FastDiv fv = make_fastdiv(static_cast<uint32_t>(vpp)), fw = make_fastdiv(static_cast<uint32_t>(ow)),
+                      fh = make_fastdiv(static_cast<uint32_t>(oh));
         const uint4 *xv = reinterpret_cast<const uint4 *>(x);
         uint4 *yv = reinterpret_cast<uint4 *>(y);
-        if (bits == 8) maxpool_vec_kernel<8><<<grid, 256, 0, st>>>(n, h, w, vpp, k, s, oh, ow, xv, yv);
-        else if (bits == 4) maxpool_vec_kernel<4><<<grid, 256, 0, st>>>(n, h, w, vpp, k, s, oh, ow, xv, yv);
-        else maxpool_vec_kernel<2><<<grid, 256, 0, st>>>(n, h, w, vpp, k, s, oh, ow, xv, yv);
+        auto go = [&](auto kern) { return launch_pdl(kern, grid, 256, 0, st, total, h, w, vpp, k, s, fv, fw, fh, xv, yv); };
+        if (k == 2)
+            return bits == 8   ? go(maxpool_vec_kernel<8, true>)
+                   : bits == 4 ? go(maxpool_vec_kernel<4, true>)
+                               : go(maxpool_vec_kernel<2, true>);
+        return bits == 8   ? go(maxpool_vec_kernel<8, false>)
+               : bits == 4 ? go(maxpool_vec_kernel<4, false>)
+                           : go(maxpool_vec_kernel<2, false>);
     } else {
         const long long total = pix * (c * bits / 8);
         const unsigned grid = static_cast<unsigned>((total + 255) / 256);
