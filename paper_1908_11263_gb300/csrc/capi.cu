@@ -434,6 +434,16 @@ qnn_status qconv_hwc_binary(const qnn_conv_desc *d, const void *x, const void *w
     s.sh = d->stride_h; s.sw = d->stride_w; s.ph = d->pad_h; s.pw = d->pad_w; s.bits = 1;
     s.oh = (d->h + 2 * d->pad_h - d->kh) / d->stride_h + 1;
     s.ow = (d->w + 2 * d->pad_w - d->kw) / d->stride_w + 1;
+    // the window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows)
+    const WinPlan wplan = plan_conv_win(s);
+    if (wplan.ok && wplan.nch_max == 1 && aligned(x, 16) && aligned(w, 16)) {
+        ConvParams p{};
+        p.x = static_cast<const uint8_t *>(x);
+        p.w = static_cast<const uint8_t *>(w);
+        p.y = static_cast<uint8_t *>(y);
+        p.thresholds = thresholds;
+        return from_cuda(launch_conv_win(wplan, s, p, static_cast<cudaStream_t>(stream)));
+    }
     return from_cuda(launch_conv_binary(s, static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), thresholds,
                                         static_cast<uint8_t *>(y), static_cast<cudaStream_t>(stream)));
 }

@@ -66,7 +66,8 @@ WinPlan plan_conv_win(const ConvShape &s)
         const int sp = win::kCols * S + (p.fold ? 0 : s.kw - 1), wh = win::kRows + s.kh - 1;
         if (wh * sp > win::kMaxKP * 128) continue;  // converter positions per thread
         const int tiles_x = (s.ow + win::kCols * S - 1) / (win::kCols * S);
-        const bool full_rows = tiles_x == 1 || p.fold;  // folded windows read whole rows
+        // folded windows read whole rows, INT-1 ones too (their pixels are no 16-byte units)
+        const bool full_rows = tiles_x == 1 || p.fold || s.bits == 1;
         const long long row_bytes = s.w * cb;
         uint32_t raw_row_bytes;
         if (full_rows) {
@@ -178,7 +179,7 @@ win::WinArgs win_args(const WinPlan &plan, const ConvShape &s, const ConvParams 
     a.kappa = p.kappa;
     a.lambda = p.lambda;
     a.shifts = p.shifts;
-    a.thr = s.thr ? p.thresholds : nullptr;
+    a.thr = s.thr || s.bits == 1 ? p.thresholds : nullptr;
     a.shift = p.shift;
     a.n = s.n; a.h = s.h; a.w_ = s.w; a.c = s.c; a.m = s.m; a.kh = s.kh; a.kw = s.kw;
     a.ph = s.ph; a.pw = s.pw; a.oh = s.oh; a.ow = s.ow;
@@ -234,6 +235,7 @@ cudaError_t launch_win(const WinPlan &plan, const ConvShape &s, const win::WinAr
     switch (s.bits) {
         case 8: return launch_win_bits<8>(a, plan.nt, grid, plan.smem_bytes, st);
         case 4: return launch_win_bits<4>(a, plan.nt, grid, plan.smem_bytes, st);
+        case 1: return launch_win_bits<1>(a, plan.nt, grid, plan.smem_bytes, st);
         default: return launch_win_bits<2>(a, plan.nt, grid, plan.smem_bytes, st);
     }
 }

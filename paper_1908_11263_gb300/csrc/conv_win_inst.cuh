@@ -8,7 +8,7 @@
 #include "conv_win.cuh"
 
 #ifndef QNN_WIN_BITS
-#error "define QNN_WIN_BITS (8, 4 or 2) before including conv_win_inst.cuh"
+#error "define QNN_WIN_BITS (8, 4, 2 or 1) before including conv_win_inst.cuh"
 #endif
 
 namespace qnn {
@@ -66,6 +66,14 @@ cudaError_t launch_win_bits<QNN_WIN_BITS>(const win::WinArgs &a, int nt, int gri
         }
     }
 #endif
+#if QNN_WIN_BITS == 1
+    switch (nt) {  // (no fused pool at INT-1)
+        case 32: return launch_one<B, 32, false>(a, grid, smem, st);
+        case 64: return launch_one<B, 64, false>(a, grid, smem, st);
+        case 128: return launch_one<B, 128, false>(a, grid, smem, st);
+        default: return cudaErrorInvalidValue;
+    }
+#else
     switch (nt) {
         case 32: return a.pool ? launch_one<B, 32, true>(a, grid, smem, st) : launch_one<B, 32, false>(a, grid, smem, st);
         case 64: return a.pool ? launch_one<B, 64, true>(a, grid, smem, st) : launch_one<B, 64, false>(a, grid, smem, st);
@@ -73,6 +81,7 @@ cudaError_t launch_win_bits<QNN_WIN_BITS>(const win::WinArgs &a, int nt, int gri
             return a.pool ? launch_one<B, 128, true>(a, grid, smem, st) : launch_one<B, 128, false>(a, grid, smem, st);
         default: return cudaErrorInvalidValue;
     }
+#endif
 }
 
 }  // namespace qnn
