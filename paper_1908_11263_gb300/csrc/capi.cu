@@ -105,50 +105,53 @@ int general_or_wide(Choice *c, const ConvShape &s)
     return c->gplan.ok ? kWide : kGeneral;
 }
 
+// The planners run in the order of preference and only as far as needed: a call
+// plans once (planning four times over cost a one-shot call about 3 us).
 Choice choose(const qnn_conv_desc *d, const ConvShape &s)
 {
-    Choice c;
-    c.plan = plan_conv_tc(s);
-    c.wplan = plan_conv_win(s);
+    Choice c{};
     switch (d->algo) {
-        case QNN_ALGO_DIRECT: c.kernel = kDirect; break;
-        case QNN_ALGO_TC_WINDOW: c.kernel = c.wplan.ok ? kWindow : -QNN_EUNSUPPORTED; break;
-        case QNN_ALGO_TC_GENERAL: c.kernel = c.plan.ok ? kGeneral : -QNN_EUNSUPPORTED; break;
-        case QNN_ALGO_TENSORCORE:
-            c.kernel = c.wplan.ok ? kWindow : c.plan.ok ? general_or_wide(&c, s) : -QNN_EUNSUPPORTED;
-            break;
-        default:
-            c.kernel = c.wplan.ok ? kWindow : c.plan.ok ? general_or_wide(&c, s) : kDirect;
-            // layers that no stride-1 kernel takes: the gather kernel on the caller's filters
-            if (c.kernel == kDirect) {
-                c.gplan = plan_conv_gather(s, 0, device_sm_count());
-                if (c.gplan.ok) c.kernel = kGather;
-            }
-            break;
+        case QNN_ALGO_DIRECT: c.kernel = kDirect; return c;
+        case QNN_ALGO_TC_GENERAL:
+            c.plan = plan_conv_tc(s);
+            c.kernel = c.plan.ok ? kGeneral : -QNN_EUNSUPPORTED;
+            return c;
+        default: break;
+    }
+    c.wplan = plan_conv_win(s);
+    if (c.wplan.ok) {
+        c.kernel = kWindow;
+        return c;
+    }
+    c.kernel = -QNN_EUNSUPPORTED;
+    if (d->algo == QNN_ALGO_TC_WINDOW) return c;
+    c.plan = plan_conv_tc(s);
+    if (c.plan.ok) {
+        c.kernel = general_or_wide(&c, s);
+    } else if (d->algo != QNN_ALGO_TENSORCORE) {
+        // layers that no stride-1 kernel takes: the gather kernel on the caller's filters
+        c.gplan = plan_conv_gather(s, 0, device_sm_count());
+        c.kernel = c.gplan.ok ? kGather : kDirect;
     }
     return c;
 }
 
 // QNN_ALGO_DIRECT or QNN_ALGO_TENSORCORE (either tensor-core kernel), or a negative status.
-int choose_algo(const qnn_conv_desc *d, const ConvShape &s, TcPlan *plan)
+int algo_of(const Choice &c)
 {
-    const Choice c = choose(d, s);
-    *plan = c.plan;
     if (c.kernel < 0) return c.kernel;
     return c.kernel == kDirect || c.kernel == kGather ? QNN_ALGO_DIRECT : QNN_ALGO_TENSORCORE;
 }
 
 qnn_status from_cuda(cudaError_t e) { return e == cudaSuccess ? QNN_OK : QNN_ECUDA; }
 
-// Filters and compression constants; also resolves the algorithm (negative = error).
-qnn_status check_params(const qnn_conv_desc *d, const ConvShape &s, const void *w, const int32_t *bias,
-                        const int16_t *kappa, const int32_t *lambda, const uint8_t *shifts, TcPlan *plan)
+// Filters and compression constants.
+qnn_status check_params(const qnn_conv_desc *d, const void *w, const int32_t *bias, const int16_t *kappa,
+                        const int32_t *lambda, const uint8_t *shifts)
 {
     if (!w || !kappa || !lambda) return QNN_EINVAL;
     if (!shifts && (d->shift < 0 || d->shift > 62)) return QNN_EINVAL;
     if (!aligned(w, 16) || !aligned(bias, 4) || !aligned(kappa, 2) || !aligned(lambda, 4)) return QNN_EALIGN;
-    const int algo = choose_algo(d, s, plan);
-    if (algo < 0) return static_cast<qnn_status>(-algo);
     return QNN_OK;
 }
 
@@ -232,8 +235,7 @@ int32_t qconv_hwc_algo(const qnn_conv_desc *d)
     ConvShape s;
     qnn_status st = check_conv(d, &s);
     if (st != QNN_OK) return -static_cast<int32_t>(st);
-    TcPlan plan;
-    return choose_algo(d, s, &plan);
+    return algo_of(choose(d, s));
 }
 
 int32_t qconv_hwc_mma_operand_bits(const qnn_conv_desc *d)
@@ -255,10 +257,11 @@ qnn_status qconv_hwc_prepare(const qnn_conv_desc *d, const void *w, const int32_
     ConvShape s;
     qnn_status st = check_conv(d, &s);
     if (st != QNN_OK) return st;
-    TcPlan plan;
-    st = check_params(d, s, w, bias, kappa, lambda, shifts, &plan);
+    st = check_params(d, w, bias, kappa, lambda, shifts);
     if (st != QNN_OK) return st;
     const Choice c = choose(d, s);
+    if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
+    const TcPlan &plan = c.plan;
     if (c.kernel == kDirect || c.kernel == kGather) return QNN_OK;
     ConvParams p{nullptr, static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts, d->shift, nullptr};
     if (c.kernel == kWindow) {
@@ -308,10 +311,11 @@ qnn_status qconv_hwc(const qnn_conv_desc *d, const void *x, const void *w, const
     if (st != QNN_OK) return st;
     if (s.n > 0 && (!x || !y)) return QNN_EINVAL;
     if (!aligned(x, 16) || !aligned(y, 16)) return QNN_EALIGN;
-    TcPlan plan;
-    st = check_params(d, s, w, bias, kappa, lambda, shifts, &plan);
+    st = check_params(d, w, bias, kappa, lambda, shifts);
     if (st != QNN_OK) return st;
     const Choice c = choose(d, s);
+    if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
+    const TcPlan &plan = c.plan;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (c.kernel == kWindow) {  // one launch; the filters are read where the caller keeps them
         ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
@@ -349,11 +353,12 @@ qnn_status qconv_hwc_pool2(const qnn_conv_desc *d, const void *x, const void *w,
     s.pool = 1;
     if (s.n > 0 && (!x || !y)) return QNN_EINVAL;
     if (!aligned(x, 16) || !aligned(y, 16)) return QNN_EALIGN;
-    TcPlan plan;
-    st = check_params(d, s, w, bias, kappa, lambda, shifts, &plan);
+    st = check_params(d, w, bias, kappa, lambda, shifts);
     if (st != QNN_OK) return st;
     // the fused pool runs in the tensor-core kernels only (strip tiles)
     const Choice c = choose(d, s);
+    if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
+    const TcPlan &plan = c.plan;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
                  d->shift, static_cast<uint8_t *>(y)};
@@ -399,15 +404,14 @@ qnn_status qconv_hwc_thresholds(const qnn_conv_desc *d, const void *x, const voi
     if (s.n > 0 && (!x || !y)) return QNN_EINVAL;
     if (!w || !thresholds) return QNN_EINVAL;
     if (!aligned(x, 16) || !aligned(y, 16) || !aligned(w, 16) || !aligned(thresholds, 4)) return QNN_EALIGN;
-    TcPlan plan;
-    const int algo = choose_algo(d, s, &plan);
-    if (algo < 0) return static_cast<qnn_status>(-algo);
     const Choice c = choose(d, s);
+    if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
+    const TcPlan &plan = c.plan;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), nullptr, nullptr, nullptr, nullptr,
                  0, static_cast<uint8_t *>(y), thresholds};
     if (c.kernel == kWindow) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-    if (algo == QNN_ALGO_TENSORCORE) {
+    if (c.kernel == kGeneral) {
         st = check_workspace(plan, workspace, workspace_bytes);
         if (st != QNN_OK) return st;
         cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, plan.nchunks);
@@ -457,11 +461,13 @@ qnn_status qconv_hwc_noalloc(const qnn_conv_desc *d, const void *x, const void *
     if (st != QNN_OK) return st;
     if (s.n > 0 && (!x || !y)) return QNN_EINVAL;
     if (!aligned(x, 16) || !aligned(y, 16)) return QNN_EALIGN;
-    TcPlan plan;
-    st = check_params(d, s, w, bias, kappa, lambda, shifts, &plan);
+    st = check_params(d, w, bias, kappa, lambda, shifts);
     if (st != QNN_OK) return st;
+    const int algo = algo_of(choose(d, s));
+    if (algo < 0) return static_cast<qnn_status>(-algo);
+    const TcPlan plan = plan_conv_tc(s);
     // this entry point runs the general tensor-core kernel, whose prepared filters go to the scratch array
-    if (choose_algo(d, s, &plan) != QNN_ALGO_TENSORCORE || !plan.ok || d->algo == QNN_ALGO_TC_WINDOW)
+    if (algo != QNN_ALGO_TENSORCORE || !plan.ok || d->algo == QNN_ALGO_TC_WINDOW)
         return QNN_EUNSUPPORTED;
     if (plan.workspace_bytes > static_cast<size_t>(QNN_NOALLOC_SCRATCH_BYTES)) return QNN_ESCRATCH;
     // an empty batch computes nothing, so it enqueues nothing and leaves the

@@ -52,6 +52,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = False):
     """Load libqnn.so (building it first only when asked)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -120,13 +122,17 @@ def _check(status: int, what: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    """The stream's handle; the current device's current stream for None (the raw handle: building
+    a Stream object for it takes longer than the rest of a call's marshalling)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dev(t: torch.Tensor, dtype, name):
@@ -143,6 +149,42 @@ def conv_desc(n, h, w, c, m, kh, kw, stride=(1, 1), pad=(0, 0), bits=8, shift=0,
     sh, sw = (stride, stride) if isinstance(stride, int) else stride
     ph, pw = (pad, pad) if isinstance(pad, int) else pad
     return ConvDesc(ctypes.sizeof(ConvDesc), n, h, w, c, m, kh, kw, sh, sw, ph, pw, bits, shift, algo)
+
+
+class _Layer:
+    """What a convolution call derives from its sizes alone: the descriptor, the output shape, the
+    workspace it needs."""
+    __slots__ = ("desc", "ref", "out_shape", "nbytes", "own_nbytes")
+
+    def __init__(self, n, h, w, c, m, kh, kw, stride, pad, bits, shift, algo):
+        self.desc = d = conv_desc(n, h, w, c, m, kh, kw, stride, pad, bits, shift, algo)
+        self.ref = ctypes.byref(d)
+        self.out_shape = (n, (h + 2 * d.pad_h - kh) // d.stride_h + 1, (w + 2 * d.pad_w - kw) // d.stride_w + 1,
+                          m * bits // 8)
+        self.nbytes = self.own_nbytes = 0
+        if bits != 1:
+            self.nbytes = workspace_size(d)
+            # the window kernel leaves the workspace of a one-shot call alone
+            self.own_nbytes = 0 if self.nbytes and tc_kernel(d) == ALGO_TC_WINDOW else self.nbytes
+
+
+_layers: dict = {}
+
+
+def _layer(*sizes) -> _Layer:
+    """The _Layer of these sizes; the last few hundred are kept (they hold no tensors)."""
+    layer = _layers.get(sizes)
+    if layer is None:
+        layer = _Layer(*sizes)
+        if len(_layers) >= 512:
+            _layers.clear()
+        _layers[sizes] = layer
+    return layer
+
+
+def _pair(v):
+    """A stride or padding as a tuple (dictionary keys take no lists)."""
+    return v if isinstance(v, int) else tuple(v)
 
 
 def workspace_size(desc: ConvDesc) -> int:
@@ -183,7 +225,8 @@ def _workspace(nbytes: int, device, stream):
     """Workspace per (device, stream): calls on one stream never overlap."""
     if nbytes == 0:
         return None
-    key = (device.index, stream.cuda_stream if stream is not None else torch.cuda.current_stream(device).cuda_stream)
+    key = (device.index,
+           stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(device.index))
     buf = _workspaces.get(key)
     if buf is None or buf.numel() < nbytes:
         buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
@@ -207,20 +250,17 @@ def conv_hwc(x, w, kappa, lam, *, bias=None, shifts=None, shift=0, bits=8, strid
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    desc = conv_desc(n, h, wd, cb * per, m, kh, kw, stride, pad, bits, shift, algo)
-    oh = (h + 2 * desc.pad_h - kh) // desc.stride_h + 1
-    ow = (wd + 2 * desc.pad_w - kw) // desc.stride_w + 1
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, _pair(stride), _pair(pad), bits, shift, algo)
     if out is None:
-        out = torch.empty((n, oh, ow, m // per), dtype=torch.uint8, device=x.device)
+        out = x.new_empty(layer.out_shape)
     else:
         _dev(out, torch.uint8, "out")
-    nbytes = workspace_size(desc)
     if workspace is None:
-        workspace = _workspace(nbytes, x.device, stream)
-    elif workspace.numel() < nbytes:
+        workspace = _workspace(layer.own_nbytes, x.device, stream)
+    elif workspace.numel() < layer.nbytes:
         raise ValueError("workspace too small")
-    st = load().qconv_hwc(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(kappa), _ptr(lam), _ptr(shifts),
-                          _ptr(out), _ptr(workspace), ctypes.c_size_t(nbytes), _stream(stream))
+    st = load().qconv_hwc(layer.ref, x.data_ptr(), w.data_ptr(), _ptr(bias), kappa.data_ptr(), lam.data_ptr(),
+                          _ptr(shifts), out.data_ptr(), _ptr(workspace), layer.nbytes, _stream(stream))
     _check(st, "qconv_hwc")
     return out
 
@@ -242,20 +282,18 @@ def conv_hwc_pool2(x, w, kappa, lam, *, bias=None, shifts=None, shift=0, bits=8,
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    desc = conv_desc(n, h, wd, cb * per, m, kh, kw, 1, pad, bits, shift, algo)
-    oh = h + 2 * desc.pad_h - kh + 1
-    ow = wd + 2 * desc.pad_w - kw + 1
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, 1, _pair(pad), bits, shift, algo)
+    _, oh, ow, mb = layer.out_shape
     if out is None:
-        out = torch.empty((n, oh // 2, ow // 2, m // per), dtype=torch.uint8, device=x.device)
+        out = x.new_empty((n, oh // 2, ow // 2, mb))
     else:
         _dev(out, torch.uint8, "out")
-    nbytes = workspace_size(desc)
     if workspace is None:
-        workspace = _workspace(nbytes, x.device, stream)
-    elif workspace.numel() < nbytes:
+        workspace = _workspace(layer.own_nbytes, x.device, stream)
+    elif workspace.numel() < layer.nbytes:
         raise ValueError("workspace too small")
-    st = load().qconv_hwc_pool2(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(kappa), _ptr(lam),
-                                _ptr(shifts), _ptr(out), _ptr(workspace), ctypes.c_size_t(nbytes), _stream(stream))
+    st = load().qconv_hwc_pool2(layer.ref, x.data_ptr(), w.data_ptr(), _ptr(bias), kappa.data_ptr(), lam.data_ptr(),
+                                _ptr(shifts), out.data_ptr(), _ptr(workspace), layer.nbytes, _stream(stream))
     _check(st, "qconv_hwc_pool2")
     return out
 
@@ -275,20 +313,18 @@ def conv_hwc_thresholds(x, w, thresholds, *, bits, stride=1, pad=0, algo=ALGO_AU
         raise ValueError("x and w disagree on the channel count")
     if tuple(thresholds.shape) != (m, (1 << bits) - 1):
         raise ValueError(f"thresholds must have shape {(m, (1 << bits) - 1)}")
-    desc = conv_desc(n, h, wd, cb * per, m, kh, kw, stride, pad, bits, 0, algo)
-    oh = (h + 2 * desc.pad_h - kh) // desc.stride_h + 1
-    ow = (wd + 2 * desc.pad_w - kw) // desc.stride_w + 1
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, _pair(stride), _pair(pad), bits, 0, algo)
     if out is None:
-        out = torch.empty((n, oh, ow, m // per), dtype=torch.uint8, device=x.device)
+        out = x.new_empty(layer.out_shape)
     else:
         _dev(out, torch.uint8, "out")
-    nbytes = workspace_size(desc)
+    # (planned with the thresholds, which take shared memory, the layer may need its workspace all the same)
     if workspace is None:
-        workspace = _workspace(nbytes, x.device, stream)
-    elif workspace.numel() < nbytes:
+        workspace = _workspace(layer.nbytes, x.device, stream)
+    elif workspace.numel() < layer.nbytes:
         raise ValueError("workspace too small")
-    st = load().qconv_hwc_thresholds(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(thresholds), _ptr(out),
-                                     _ptr(workspace), ctypes.c_size_t(nbytes), _stream(stream))
+    st = load().qconv_hwc_thresholds(layer.ref, x.data_ptr(), w.data_ptr(), thresholds.data_ptr(), out.data_ptr(),
+                                     _ptr(workspace), layer.nbytes, _stream(stream))
     _check(st, "qconv_hwc_thresholds")
     return out
 
@@ -303,15 +339,13 @@ def conv_binary(x, w, thresholds, *, stride=1, pad=0, out=None, stream=None):
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    desc = conv_desc(n, h, wd, cb * 8, m, kh, kw, stride, pad, 1, 0, ALGO_AUTO)
-    oh = (h + 2 * desc.pad_h - kh) // desc.stride_h + 1
-    ow = (wd + 2 * desc.pad_w - kw) // desc.stride_w + 1
+    layer = _layer(n, h, wd, cb * 8, m, kh, kw, _pair(stride), _pair(pad), 1, 0, ALGO_AUTO)
     if out is None:
-        out = torch.empty((n, oh, ow, m // 8), dtype=torch.uint8, device=x.device)
+        out = x.new_empty(layer.out_shape)
     else:
         _dev(out, torch.uint8, "out")
-    _check(load().qconv_hwc_binary(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(thresholds), _ptr(out), _stream(stream)),
-           "qconv_hwc_binary")
+    _check(load().qconv_hwc_binary(layer.ref, x.data_ptr(), w.data_ptr(), thresholds.data_ptr(), out.data_ptr(),
+                                   _stream(stream)), "qconv_hwc_binary")
     return out
 
 
@@ -381,9 +415,9 @@ class PreparedConv:
     def __call__(self, x, out=None, stream=None):
         _dev(x, torch.uint8, "x")
         if out is None:
-            out = torch.empty(self.out_shape, dtype=torch.uint8, device=x.device)
-        st = load().qconv_hwc_run(ctypes.byref(self.desc), _ptr(x), _ptr(out), _ptr(self.workspace),
-                                  ctypes.c_size_t(self.nbytes), _stream(stream))
+            out = x.new_empty(self.out_shape)
+        st = load().qconv_hwc_run(ctypes.byref(self.desc), x.data_ptr(), out.data_ptr(), self.workspace.data_ptr(),
+                                  self.nbytes, _stream(stream))
         _check(st, "qconv_hwc_run")
         return out
 
@@ -393,9 +427,9 @@ class PreparedConv:
         _dev(x, torch.uint8, "x")
         if out is None:
             n, _, _, mb = self.out_shape
-            out = torch.empty((n, self.oh // 2, self.ow // 2, mb), dtype=torch.uint8, device=x.device)
-        st = load().qconv_hwc_pool2_run(ctypes.byref(self.desc), _ptr(x), _ptr(out), _ptr(self.workspace),
-                                        ctypes.c_size_t(self.nbytes), _stream(stream))
+            out = x.new_empty((n, self.oh // 2, self.ow // 2, mb))
+        st = load().qconv_hwc_pool2_run(ctypes.byref(self.desc), x.data_ptr(), out.data_ptr(),
+                                        self.workspace.data_ptr(), self.nbytes, _stream(stream))
         _check(st, "qconv_hwc_pool2_run")
         return out
 
@@ -424,7 +458,7 @@ def maxpool(x, k=2, s=2, bits=8, *, out=None, stream=None):
     c = cb * 8 // bits
     oh, ow = (h - k) // s + 1, (wd - k) // s + 1
     if out is None:
-        out = torch.empty((n, oh, ow, cb), dtype=torch.uint8, device=x.device)
+        out = x.new_empty((n, oh, ow, cb))
     st = load().qmaxpool(n, h, wd, c, k, s, bits, _ptr(x), _ptr(out), _stream(stream))
     _check(st, "qmaxpool")
     return out
