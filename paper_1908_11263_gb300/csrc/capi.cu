@@ -86,8 +86,12 @@ qnn_status check_conv(const qnn_conv_desc *d, ConvShape *s)
 // QNN_ALGO_TC_GENERAL force one of them.  INT-8 layers that no prepared kernel
 // takes run on the gather kernel with the caller's filters (3 to 80 times as
 // fast as the CUDA-core kernel); they are reported as QNN_ALGO_DIRECT, need no
-// workspace and cannot be prepared.
-enum Kernel { kDirect = 1, kWindow = 3, kGeneral = 4, kGather = 5, kWide = 6 };
+// workspace and cannot be prepared.  One-shot calls of layers left to the general
+// kernel whose pixels are no whole 16-byte units run on the window kernel with
+// windows read as whole image rows (INT-2 staircase, 34 x 32 x 32 -> 16, batch
+// 1,453: 83.9 us, 200.9 on the general kernel);
+// they keep the general kernel's workspace rules and preparation.
+enum Kernel { kDirect = 1, kWindow = 3, kGeneral = 4, kGather = 5, kWide = 6, kRows = 7 };
 
 struct Choice {
     int kernel;  // Kernel, or a negative qnn_status
@@ -128,9 +132,18 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
     c.plan = plan_conv_tc(s);
     if (c.plan.ok) {
         c.kernel = general_or_wide(&c, s);
+        if (c.kernel == kGeneral) {
+            // one-shot calls: the window kernel on windows read as whole image rows
+            c.wplan = plan_conv_win(s, true);
+            if (c.wplan.ok) c.kernel = kRows;
+        }
     } else if (d->algo != QNN_ALGO_TENSORCORE) {
         // layers that no stride-1 kernel takes: the gather kernel on the caller's filters
-        c.gplan = plan_conv_gather(s, 0, device_sm_count());
+        // (a few products per output, and few outputs: the CUDA-core kernel has no pipeline to fill; 7 images of
+        // 37 x 18 x 3 -> 160, 1 x 1 stride 2, take it 3.6 us, the gather kernel 6.0)
+        const long long k = static_cast<long long>(s.kh) * s.kw * s.c;
+        const bool tiny = k <= 8 && k * s.n * s.oh * s.ow * s.m <= (4ll << 20);
+        if (!tiny) c.gplan = plan_conv_gather(s, 0, device_sm_count());
         c.kernel = c.gplan.ok ? kGather : kDirect;
     }
     return c;
@@ -215,7 +228,7 @@ qnn_status qconv_hwc_workspace_size(const qnn_conv_desc *d, size_t *bytes)
     const Choice c = choose(d, s);
     if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
     *bytes = c.kernel == kWindow                          ? c.wplan.img_bytes
-             : c.kernel == kGeneral || c.kernel == kWide ? c.plan.workspace_bytes
+             : c.kernel == kGeneral || c.kernel == kWide || c.kernel == kRows ? c.plan.workspace_bytes
                                                           : 0;
     return QNN_OK;
 }
@@ -227,7 +240,7 @@ int32_t qconv_hwc_tc_kernel(const qnn_conv_desc *d)
     if (st != QNN_OK) return -static_cast<int32_t>(st);
     const Choice c = choose(d, s);
     if (c.kernel < 0) return c.kernel;
-    return c.kernel == kWindow ? kWindow : c.kernel == kGeneral || c.kernel == kWide ? kGeneral : 0;
+    return c.kernel == kWindow ? kWindow : c.kernel == kGeneral || c.kernel == kWide || c.kernel == kRows ? kGeneral : 0;
 }
 
 int32_t qconv_hwc_algo(const qnn_conv_desc *d)
@@ -246,7 +259,7 @@ int32_t qconv_hwc_mma_operand_bits(const qnn_conv_desc *d)
     const Choice c = choose(d, s);
     if (c.kernel < 0) return c.kernel;
     if (c.kernel == kWindow) return c.wplan.fp8 ? 8 : 16;
-    if (c.kernel == kGeneral || c.kernel == kWide) return c.plan.fp8 ? 8 : 16;
+    if (c.kernel == kGeneral || c.kernel == kWide || c.kernel == kRows) return c.plan.fp8 ? 8 : 16;
     return 0;
 }
 
@@ -322,11 +335,12 @@ qnn_status qconv_hwc(const qnn_conv_desc *d, const void *x, const void *w, const
                      d->shift, static_cast<uint8_t *>(y)};
         return from_cuda(launch_conv_win(c.wplan, s, p, cs));
     }
-    if (c.kernel == kGeneral || c.kernel == kWide) {
+    if (c.kernel == kGeneral || c.kernel == kWide || c.kernel == kRows) {
         st = check_workspace(plan, workspace, workspace_bytes);
         if (st != QNN_OK) return st;
         ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
                      d->shift, static_cast<uint8_t *>(y)};
+        if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
         cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, c.kernel == kWide ? 0 : plan.nchunks);
         if (e != cudaSuccess) return QNN_ECUDA;
         if (c.kernel == kWide)
@@ -363,9 +377,10 @@ qnn_status qconv_hwc_pool2(const qnn_conv_desc *d, const void *x, const void *w,
     ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
                  d->shift, static_cast<uint8_t *>(y)};
     if (c.kernel == kWindow) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-    if (c.kernel != kGeneral || !plan.strip) return QNN_EUNSUPPORTED;
+    if ((c.kernel != kGeneral && c.kernel != kRows) || !plan.strip) return QNN_EUNSUPPORTED;
     st = check_workspace(plan, workspace, workspace_bytes);
     if (st != QNN_OK) return st;
+    if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
     cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, plan.nchunks);
     if (e == cudaSuccess) e = launch_conv_tc_run(plan, s, p.x, p.y, workspace, cs, true);
     return from_cuda(e);
@@ -411,9 +426,10 @@ qnn_status qconv_hwc_thresholds(const qnn_conv_desc *d, const void *x, const voi
     ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), nullptr, nullptr, nullptr, nullptr,
                  0, static_cast<uint8_t *>(y), thresholds};
     if (c.kernel == kWindow) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-    if (c.kernel == kGeneral) {
+    if (c.kernel == kGeneral || c.kernel == kRows) {
         st = check_workspace(plan, workspace, workspace_bytes);
         if (st != QNN_OK) return st;
+        if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
         cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, plan.nchunks);
         if (e == cudaSuccess) e = launch_conv_tc_run(plan, s, p.x, p.y, workspace, cs, true);
         return from_cuda(e);
@@ -438,8 +454,11 @@ qnn_status qconv_hwc_binary(const qnn_conv_desc *d, const void *x, const void *w
     s.sh = d->stride_h; s.sw = d->stride_w; s.ph = d->pad_h; s.pw = d->pad_w; s.bits = 1;
     s.oh = (d->h + 2 * d->pad_h - d->kh) / d->stride_h + 1;
     s.ow = (d->w + 2 * d->pad_w - d->kw) / d->stride_w + 1;
-    // the window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows)
-    const WinPlan wplan = plan_conv_win(s);
+    // The window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows), from
+    // 128 products per output on: below that the counts are few (209 images of 7 x 20 x 32 -> 88, 1 x 1: 6.8 us
+    // with counts, 11.5 there; 299 of 30 x 28 x 64 -> 104, 1 x 1: 21.7 and 20.6; 3 x 3 layers of 32 channels 26.4 and 9.7)
+    const bool many = static_cast<long long>(s.kh) * s.kw * s.c >= 128;
+    const WinPlan wplan = many ? plan_conv_win(s) : WinPlan{};
     if (wplan.ok && wplan.nch_max == 1 && aligned(x, 16) && aligned(w, 16)) {
         ConvParams p{};
         p.x = static_cast<const uint8_t *>(x);

@@ -54,12 +54,13 @@
 // bulk copies of the fp16 filters that conv_tc_prep_kernel laid out.
 //
 // Measured per call (was: general tensor-core kernel for the first three, CUDA
-// cores for the others): 28 x 28 x 128 -> 128 3 x 3, batch 64: 16.3 us (49.2);
-// 14 x 14 x 256 -> 256 3 x 3: 15.9 us (47.3); 14 x 14 x 256 -> 512 1 x 1: 12.3 us
-// (30.7); 56 x 56 x 64 -> 128 3 x 3 stride 2: 20.1 us (1,627); 33 x 45 x 20 -> 44
-// 3 x 3, batch 37: 25.5 us (75.5).  The flat-window layers are bound by the MMA
-// warp's issue (an item of four N = 192 MMAs takes 550 cycles, 384 without any
-// wait); im2col layers by the latency of the producers' global loads.
+// cores for the others): 28 x 28 x 128 -> 128 3 x 3, batch 64: 16.1 us (49.2);
+// 14 x 14 x 256 -> 256 3 x 3: 15.8 us (47.3); 14 x 14 x 256 -> 512 1 x 1: 12.1 us
+// (30.7); 56 x 56 x 64 -> 128 3 x 3 stride 2: 19.9 us (1,627); 33 x 45 x 20 -> 44
+// 3 x 3, batch 37: 16.9 us (70; 25.4 with a branch per word of an unaligned
+// granule).  The flat-window layers are bound by the MMA warp's issue (an item of
+// four N = 192 MMAs takes 550 cycles, 384 without any wait); im2col layers by the
+// latency of the producers' global loads.
 //
 // Warp roles (one persistent CTA per SM, 18 warps):
 //   warps 0-7    producers: global memory -> registers -> staged fp16
@@ -86,6 +87,7 @@ constexpr int kSlabGran = 4;         // granules (MMA k-steps) per stage
 constexpr int kMaxStages = 8, kMaxW = 9, kMaxSlots = 4;
 constexpr int kChunkGranules = 64;   // 64 * 16 products of at most 2^14: 2^24
 constexpr int kChunkAbs = 1 << 17;   // 128 * sum |w| <= 2^24
+constexpr int kTabled = 256;         // granules whose place is tabulated
 constexpr int kMaxAbs = 16;          // stages whose sums of |w| a prepared layer carries
 constexpr int kMaxIter = 8;          // pixels per producer thread and stage
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB opt-in dynamic shared memory per block
@@ -137,6 +139,7 @@ struct Shared {
     uint32_t tmem;
     int abs_max[kMaxAbs];
     int sums[2][kRowsW];    // per filter: positive part, negative part
+    int4 gran[kTabled];     // im2col: kernel row, first byte in it, kernel column, input offset of a granule
 };
 
 // One 16-byte granule as loaded: whole (aligned kernels) or the five words it
@@ -161,26 +164,28 @@ struct Gran<false> {
         for (int k = 0; k < 5; ++k) q[k] = 0;
         meta = 0;
     }
-    // bytes [lo, hi) of the 16 at p (any alignment); no word outside the ones these
-    // bytes lie in is read, nor one that reaches past `end`
-    __device__ __forceinline__ void load(const uint8_t *p, int lo, int hi, const uint8_t *end)
+    // bytes [lo, hi) of the 16 at p (any alignment) of the tensor [begin, end): the
+    // five aligned words around them, read whole where all lie inside the tensor,
+    // else only what overlaps the bytes (one branch, taken at the tensor's ends)
+    __device__ __forceinline__ void load(const uint8_t *p, int lo, int hi, const uint8_t *begin, const uint8_t *end)
     {
         const uint32_t sh = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p) & 3u);
         const uint8_t *a = p - sh;
+        meta = (sh * 8u) | static_cast<uint32_t>(lo) << 8 | static_cast<uint32_t>(max(lo, hi)) << 16;
+        if (hi > lo && a >= begin && a + 20 <= end) {
+            const uint32_t *q4 = reinterpret_cast<const uint32_t *>(a);
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = __ldg(q4 + k);
+            return;
+        }
         const int b0 = lo + static_cast<int>(sh), b1 = hi + static_cast<int>(sh);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            q[k] = 0;
-            if (4 * k + 4 > b0 && 4 * k < b1 && hi > lo) {
-                if (a + 4 * k + 4 <= end) {
-                    q[k] = __ldg(reinterpret_cast<const uint32_t *>(a + 4 * k));
-                } else {  // the tensor's last word, when its bytes are not whole words
-                    for (int b = 0; b < 4; ++b)
-                        if (a + 4 * k + b < end) q[k] |= static_cast<uint32_t>(__ldg(a + 4 * k + b)) << (8 * b);
-                }
-            }
+        for (int k = 0; k < 5; ++k) q[k] = 0;
+        if (hi > lo) {
+#pragma unroll
+            for (int b = 0; b < 20; ++b)
+                if (b >= b0 && b < b1) q[b / 4] |= static_cast<uint32_t>(__ldg(a + b)) << (8 * (b % 4));
         }
-        meta = (sh * 8u) | static_cast<uint32_t>(lo) << 8 | static_cast<uint32_t>(max(lo, hi)) << 16;
     }
     __device__ __forceinline__ uint4 get() const
     {
@@ -188,8 +193,10 @@ struct Gran<false> {
         const int lo = static_cast<int>((meta >> 8) & 0xFFu), hi = static_cast<int>(meta >> 16);
         uint32_t r[4];
 #pragma unroll
+        for (int k = 0; k < 4; ++k) r[k] = __funnelshift_r(q[k], q[k + 1], sh);
+        if (lo == 0 && hi == 16) return make_uint4(r[0], r[1], r[2], r[3]);
+#pragma unroll
         for (int k = 0; k < 4; ++k) {
-            r[k] = __funnelshift_r(q[k], q[k + 1], sh);
             // keep bytes [lo, hi) of the granule: byte b of word k is byte 4k + b
             const int l = min(max(lo - 4 * k, 0), 4), e = min(max(hi - 4 * k, 0), 4);
             const uint32_t below_e = e == 4 ? 0xFFFFFFFFu : (1u << (8 * e)) - 1u;
@@ -221,7 +228,7 @@ __device__ __forceinline__ void fetch_w(const Args &a, int o, int g, Gran<ALIGNE
     const int i = fdiv(g, a.fd_gr), r = (g - i * static_cast<int>(a.fd_gr.d)) * 16;
     const uint8_t *p = a.w + static_cast<uint32_t>((o * a.kh + i) * a.kwc + r);
     if constexpr (ALIGNED) v.v = __ldg(reinterpret_cast<const uint4 *>(p));
-    else v.load(p, 0, min(16, a.kwc - r), a.w + a.wbytes);
+    else v.load(p, 0, min(16, a.kwc - r), a.w, a.w + a.wbytes);
 }
 
 // Sums of the positive and the negative weights of a granule.
@@ -365,15 +372,25 @@ __device__ __forceinline__ void decode_pixels(const Args &a, int mtile, int row0
     }
 }
 
+// Where granule g lies: kernel row i, byte r of it, kernel column j (aligned
+// kernels), offset from the window's origin.
+__device__ __forceinline__ int4 gran_place(const Args &a, int g)
+{
+    const int i = fdiv(g, a.fd_gr), r = (g - i * static_cast<int>(a.fd_gr.d)) * 16;
+    return make_int4(i, r, fdiv(r, a.fd_c), i * a.row_c + r);
+}
+
 // Granule g of the thread's pixels.
 template <bool ALIGNED, int ITER>
-__device__ __forceinline__ void fetch_x(const Args &a, const Pixels &px, int g, Gran<ALIGNED> (&v)[ITER])
+__device__ __forceinline__ void fetch_x(const Args &a, const Shared *sh, const Pixels &px, int g,
+                                        Gran<ALIGNED> (&v)[ITER])
 {
     const bool in = g < a.cgr;
-    const int i = fdiv(g, a.fd_gr), r = (g - i * static_cast<int>(a.fd_gr.d)) * 16;
-    const uint32_t off = static_cast<uint32_t>(i) * static_cast<uint32_t>(a.row_c) + static_cast<uint32_t>(r);
+    const int4 place = a.cgr <= kTabled ? sh->gran[min(g, kTabled - 1)] : gran_place(a, g);
+    const int i = place.x, r = place.y;
+    const uint32_t off = static_cast<uint32_t>(place.w);
     if constexpr (ALIGNED) {
-        const int j = fdiv(r, a.fd_c);
+        const int j = place.z;
 #pragma unroll
         for (int it = 0; it < ITER; ++it) {
             const bool ok = in && static_cast<unsigned>(px.iy[it] + i) < static_cast<unsigned>(a.h) &&
@@ -387,9 +404,10 @@ __device__ __forceinline__ void fetch_x(const Args &a, const Pixels &px, int g, 
             // bytes of the kernel row inside the image: [-ix * c, (w - ix) * c), cut to the granule
             const bool row_ok = in && static_cast<unsigned>(px.iy[it] + i) < static_cast<unsigned>(a.h);
             const int lo = min(16, max(0, -px.ix[it] * a.c - r));
-            const int hi = row_ok ? max(0, min(16, min(a.kwc, (a.w_ - px.ix[it]) * a.c) - r)) : 0;
+            // (what lies past the kernel row's end meets zero filter values)
+            const int hi = row_ok && r < a.kwc ? max(0, min(16, (a.w_ - px.ix[it]) * a.c - r)) : 0;
             // (the offset of byte lo is a true one; the granule's own start may lie before the input)
-            v[it].load(a.x + static_cast<uint32_t>(px.base[it] + off + static_cast<uint32_t>(lo)) - lo, lo, hi,
+            v[it].load(a.x + static_cast<uint32_t>(px.base[it] + off + static_cast<uint32_t>(lo)) - lo, lo, hi, a.x,
                        a.x + a.xbytes);
         }
     }
@@ -421,14 +439,14 @@ __device__ __forceinline__ void produce_x(const Args &a, uint8_t *smem, Shared *
     Pixels px;
     decode_pixels<ITER>(a, mt, row0, px);
     Gran<ALIGNED> va[ITER], vb[ITER];
-    fetch_x<ALIGNED, ITER>(a, px, s * kSlabGran + q, va);
+    fetch_x<ALIGNED, ITER>(a, sh, px, s * kSlabGran + q, va);
     auto turn = [&](Gran<ALIGNED>(&use)[ITER], Gran<ALIGNED>(&load)[ITER]) {
         s += step;
         const bool moved = settle();
         const bool more = mt < a.mtiles;
         if (more) {
             if (moved) decode_pixels<ITER>(a, mt, row0, px);
-            fetch_x<ALIGNED, ITER>(a, px, s * kSlabGran + q, load);
+            fetch_x<ALIGNED, ITER>(a, sh, px, s * kSlabGran + q, load);
         }
         if (!mbar_wait_warp(&sh->x_empty[stage], ph ^ 1u, a.status)) return false;
         const uint32_t dst = dst0 + stage * a.stage_bytes;
@@ -1073,6 +1091,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_gather_kernel(const Args a)
     } else if (warp < kProdWarps) {
         if (threadIdx.x < kMaxAbs) sh->abs_max[threadIdx.x] = 0;
         sh->sums[threadIdx.x / kRowsW][threadIdx.x % kRowsW] = 0;
+    } else if (XMODE == kIm2col && warp < kEpiWarp0 + kEpiWarps) {
+        const int g = static_cast<int>(threadIdx.x) - kEpiWarp0 * 32;  // kTabled threads
+        if (g < a.cgr) sh->gran[g] = gran_place(a, g);
     }
     tc_fence_before();
     __syncthreads();

@@ -26,7 +26,7 @@ int strips_per_tile(int ow)
 
 }  // namespace
 
-WinPlan plan_conv_win(const ConvShape &s)
+WinPlan plan_conv_win(const ConvShape &s, bool rows)
 {
     WinPlan p{};
     p.ok = false;
@@ -67,7 +67,7 @@ WinPlan plan_conv_win(const ConvShape &s)
         if (wh * sp > win::kMaxKP * 128) continue;  // converter positions per thread
         const int tiles_x = (s.ow + win::kCols * S - 1) / (win::kCols * S);
         // folded windows read whole rows, INT-1 ones too (their pixels are no 16-byte units)
-        const bool full_rows = tiles_x == 1 || p.fold || s.bits == 1;
+        const bool full_rows = tiles_x == 1 || p.fold || s.bits == 1 || rows;
         const long long row_bytes = s.w * cb;
         uint32_t raw_row_bytes;
         if (full_rows) {

@@ -111,7 +111,9 @@ struct WinPlan {
     size_t img_bytes;     // qconv_hwc_prepare workspace: the prepared image (B, then the tail)
 };
 
-WinPlan plan_conv_win(const ConvShape &s);
+// rows: every window is read as whole image rows, so that pixels need not be
+// whole 16-byte units (rows still have to be) where tiles are narrower than rows.
+WinPlan plan_conv_win(const ConvShape &s, bool rows = false);
 // One launch of the window kernel.  With img == nullptr it prepares the
 // caller's filters and constants (p.w, p.bias, ...) itself; with img it reads
 // the image qconv_hwc_prepare wrote (img_bytes at img) and p carries only x, y.

@@ -86,7 +86,7 @@ static void check(const ConvShape &s, int w_rows, std::mt19937 &rng)
         CHECK(p.stage_bytes >= x_bytes + p.item_w);
     }
     CHECK(p.off_bar >= p.off_x + p.stages * p.stage_bytes && p.off_bar % 8 == 0);
-    CHECK(p.smem_bytes <= 232448 && p.smem_bytes >= p.off_bar + 1440);
+    CHECK(p.smem_bytes <= 232448 && p.smem_bytes >= p.off_bar + 1440 + 256 * 16);
     // the MMA reads 128 filter rows of every plane, laid out or not
     const long long last_w = p.resident ? items : prepared ? p.w_slots : 0;
     if (last_w) CHECK((last_w - 1) * p.item_w + 7ll * p.plane_w + 128 * 16 <= p.smem_bytes);
@@ -141,7 +141,7 @@ static void check(const ConvShape &s, int w_rows, std::mt19937 &rng)
                         CHECK((1ll * o * s.kh + i) * kwc + r + 16 <= static_cast<long long>(w.size()));
                     } else {
                         const int lo = std::min(16, std::max(0, -ix * s.c - r));
-                        const int hi = row_ok ? std::max(0, std::min(16, std::min(kwc, (s.w - ix) * s.c) - r)) : 0;
+                        const int hi = row_ok && r < kwc ? std::max(0, std::min(16, (s.w - ix) * s.c - r)) : 0;
                         granule(x, base + 1ll * i * row_c + r, lo, hi, xa);
                     }
                     granule(w, (1ll * o * s.kh + i) * kwc + r, 0, std::min(16, kwc - r), wa);

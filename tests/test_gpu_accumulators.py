@@ -96,3 +96,45 @@ def test_staircase_orders(bits, m, order):
     check_guard(buf)
     want = oracle.pack((thr[None, :, :] <= acc[:, :, None]).sum(axis=2).reshape(-1), bits)
     assert first_mismatch(out.cpu().numpy().reshape(-1), want) is None
+
+
+# (n, h, w, c, m, k, pad, bits): several tiles across rows whose pixels are no whole 16-byte units
+ROWS = [
+    (2, 18, 32, 32, 16, 3, 1, 2),
+    (1, 33, 40, 32, 104, 1, 0, 2),
+    (1, 9, 36, 96, 24, 3, 1, 2),
+    (2, 17, 22, 24, 40, 3, 1, 8),
+    (1, 20, 66, 8, 128, 5, 2, 8),
+    (3, 7, 34, 40, 64, 3, 0, 8),
+]
+
+
+@pytest.mark.parametrize("layer", ROWS, ids=lambda s: "x".join(str(v) for v in s))
+def test_windows_of_whole_rows(layer):
+    """One-shot calls, plain, with the fused pool and with thresholds, against the oracle."""
+    n, h, w, c, m, k, pad, bits = layer
+    rng = np.random.default_rng(sum(layer))
+    top, half, per = (1 << bits) - 1, 1 << (bits - 1), 8 // bits
+    x = rng.integers(0, top + 1, size=(n, h, w, c))
+    wt = rng.integers(-half, half, size=(m, k, k, c))
+    acc = oracle.conv_acc(x, wt, (1, 1), (pad, pad)).reshape(-1, m)
+    bias = (-acc.mean(axis=0)).astype(np.int32)
+    kappa = rng.integers(1, 65, size=m).astype(np.int16)
+    lam = rng.integers(-16, 17, size=m).astype(np.int32)
+    shift = max(0, int(np.ceil(np.log2(1.6 * acc.std() * 32 / top))))
+    want = conv_oracle(x, wt, bias, kappa, lam, None, shift, bits, (1, 1), (pad, pad))
+    got = conv_gpu(x, wt, bias, kappa, lam, None, shift, bits, (1, 1), (pad, pad), qnn.ALGO_AUTO)
+    assert first_mismatch(got, want) is None, first_mismatch(got, want)
+    xd = pack_gpu(x, bits).view(n, h, w, c // per)
+    wd = pack_gpu(wt, bits).view(m, k, k, c // per)
+    oh, ow = h + 2 * pad - k + 1, w + 2 * pad - k + 1
+    pooled = qnn.conv_hwc_pool2(xd, wd.view(torch.int8) if bits == 8 else wd, to_dev(kappa, torch.int16),
+                                to_dev(lam, torch.int32), bias=to_dev(bias, torch.int32), shift=shift, bits=bits, pad=pad)
+    want2 = oracle.maxpool(want, n, oh, ow, m, 2, 2, bits)
+    assert first_mismatch(pooled.cpu().numpy().reshape(-1), want2) is None
+    if bits < 8:
+        thr = np.stack([np.quantile(acc, (q + 0.5) / top, axis=0) for q in range(top)], axis=1).astype(np.int32)
+        out = qnn.conv_hwc_thresholds(xd, wd, to_dev(thr, torch.int32), bits=bits, pad=pad)
+        want3 = oracle.pack((thr[None, :, :] <= acc[:, :, None]).sum(axis=2).reshape(-1), bits)
+        assert first_mismatch(out.cpu().numpy().reshape(-1), want3) is None
+    qnn.device_status()
