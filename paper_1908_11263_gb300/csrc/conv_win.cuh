@@ -476,8 +476,8 @@ template <int KH, int KW, int KS, int S, int NT, bool F8, bool START>
 __device__ __forceinline__ void issue_fixed(uint32_t d0, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                             uint32_t idesc, int sp, uint32_t kstep_a)
 {
-    // one kernel row per iteration: its KW * KS * S MMAs unrolled
-#pragma unroll 1
+    // one kernel row per iteration: its KW * KS * S MMAs unrolled (a folded layer's rows all at once)
+#pragma unroll(KW == 1 ? KH : 1)
     for (int i = 0; i < KH; ++i) {
         const uint32_t arow = alo + static_cast<uint32_t>(i * sp);
 #pragma unroll
@@ -496,7 +496,7 @@ __device__ __forceinline__ void issue_fixed(uint32_t d0, uint32_t alo, uint32_t 
     }
 }
 
-template <int NT, bool F8>
+template <int NT, bool F8, bool FOLD>
 __device__ __forceinline__ void mma_role(const WinArgs &a, uint8_t *smem, uint64_t *a_full, uint64_t *a_empty,
                                          uint64_t *acc_full, uint64_t *acc_empty, uint64_t *done, const Misc *misc)
 {
@@ -521,7 +521,10 @@ __device__ __forceinline__ void mma_role(const WinArgs &a, uint8_t *smem, uint64
     const uint2 *tab = reinterpret_cast<const uint2 *>(smem + a.off_mtab);
     const int nu = static_cast<int>(misc->nmma);
     // the common shapes with one exact chunk issue from unrolled code
+    // (folded kernel columns: one MMA per kernel row and strip; the 32 x 32 x 3 -> 32 5 x 5
+    // layer's 12 took 2,000 cycles from the table)
     const int fixed = nch != 1 ? 0
+                      : FOLD ? (a.ksteps != 1 || a.s != 2 ? 0 : a.kh == 5 ? 6 : a.kh == 3 ? 7 : 0)
                       : (a.kh == 3 && a.kwf == 3 && a.ksteps == 2 && a.s == 2) ? 1
                       : (a.kh == 3 && a.kwf == 3 && a.ksteps == 1 && a.s == 2) ? 2
                       : (a.kh == 5 && a.kwf == 5 && a.ksteps == 2 && a.s == 2) ? 3
@@ -543,8 +546,16 @@ __device__ __forceinline__ void mma_role(const WinArgs &a, uint8_t *smem, uint64
         // (no staging but INT-8's goes without the pre-load)
         constexpr bool kStart = !F8;
         switch (fixed * 2 + (keep ? 0 : 1)) {
+            // (not compiled into the other layers' kernels, nor theirs into these)
+#define QNN_FOLDED(KH)                                                                                  \
+    if constexpr (FOLD) issue_fixed<KH, 1, 1, 2, NT, F8, false>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); \
+    break
+            case 12: QNN_FOLDED(5);
+            case 14: QNN_FOLDED(3);
+#undef QNN_FOLDED
 #define QNN_ISSUE(KH, KW, KS, S, ST) \
-    issue_fixed<KH, KW, KS, S, NT, F8, ST>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); break
+    if constexpr (!FOLD) issue_fixed<KH, KW, KS, S, NT, F8, ST>(d0, alo, ahi, blo, bhi, idesc, a.sp, kstep_a); \
+    break
             case 2: QNN_ISSUE(3, 3, 2, 2, false);
             case 4: QNN_ISSUE(3, 3, 1, 2, false);
             case 6: QNN_ISSUE(5, 5, 2, 2, false);
@@ -996,40 +1007,6 @@ __device__ __forceinline__ void pack_values(const int (&y)[G], uint32_t (&packed
     }
 }
 
-// One block of EB output channels of one strip's pixel: packed Q-bit values,
-// max-pooled over the 2x2 window when POOL (every lane shuffles), stored.
-template <int BITS, int EB, bool POOL>
-__device__ __forceinline__ void store_block(const int (&y)[EB], bool store, int valid, uint8_t *dst)
-{
-    uint32_t pk[(EB * BITS + 31) / 32];
-    pack_values<BITS, EB>(y, pk);
-    if constexpr (POOL) {
-#pragma unroll
-        for (int wd = 0; wd < (EB * BITS + 31) / 32; ++wd) {
-            pk[wd] = max_fields<BITS>(pk[wd], __shfl_xor_sync(0xffffffffu, pk[wd], 1));
-            pk[wd] = max_fields<BITS>(pk[wd], __shfl_xor_sync(0xffffffffu, pk[wd], 8));
-        }
-    }
-    if (store) store_packed<BITS, EB>(pk, valid, dst);
-}
-
-// HB packed Q-bit values of one strip's pixel (whole words when HB * Q is a
-// multiple of 32, else the low bits of one word): max-pooled over the 2x2
-// window when POOL (every lane shuffles), stored.
-template <int BITS, int HB, bool POOL>
-__device__ __forceinline__ void store_words(uint32_t (&pk)[(HB * BITS + 31) / 32 < 1 ? 1 : (HB * BITS + 31) / 32],
-                                            bool store, int valid, uint8_t *dst)
-{
-    if constexpr (POOL) {
-#pragma unroll
-        for (int wd = 0; wd < (HB * BITS + 31) / 32; ++wd) {
-            pk[wd] = max_fields<BITS>(pk[wd], __shfl_xor_sync(0xffffffffu, pk[wd], 1));
-            pk[wd] = max_fields<BITS>(pk[wd], __shfl_xor_sync(0xffffffffu, pk[wd], 8));
-        }
-    }
-    if (store) store_packed<BITS, HB>(pk, valid, dst);
-}
-
 // How a warp's channels are compressed.  Each kind has its own copy of the
 // block loop, so that the registers of the others do not weigh on it (with the
 // kinds told apart inside one loop the INT-2 layer at batch 2,048 spilled and
@@ -1057,6 +1034,38 @@ struct EpiTile {
     uint64_t *acc_empty;
     uint32_t cst_addr; // TMEM address of lam2 of channel col0 in this warp's lanes (kappa NT columns on)
 };
+
+// HB packed channels of the tile's two strips (pk0, pk1), max-pooled over the 2x2
+// window of lanes L, L^1, L^8, L^9 and stored.  Each step halves what a lane
+// keeps instead of leaving both partners with the same maximum: across the two
+// columns a lane keeps one strip (its low bit) and hands over the other, across
+// the two rows it keeps one of two words (bit 3), so a block of 8 INT-8 channels
+// takes 3 shuffles and maxima instead of 8, and all lanes store a word each.  (32 x
+// 32 x 3 -> 32, 5 x 5, batch 1,024: 44.7 -> 37.6 us with this, the cheaper INT-8
+// maximum and the unrolled issue; the CIFAR-shaped network 99.5 -> 90.1.)
+template <int BITS, int HB>
+__device__ __forceinline__ void store_pooled(const uint32_t (&pk0)[(HB * BITS + 31) / 32],
+                                             const uint32_t (&pk1)[(HB * BITS + 31) / 32], const EpiTile &e, int m0,
+                                             int valid)
+{
+    constexpr int kWords = (HB * BITS + 31) / 32;
+    static_assert(kWords <= 2, "a lane keeps one word");
+    const bool right = e.lane & 1, below = e.lane & 8;
+    uint32_t t[kWords];
+#pragma unroll
+    for (int wd = 0; wd < kWords; ++wd) {
+        const uint32_t keep = e.two && right ? pk1[wd] : pk0[wd], give = e.two && !right ? pk1[wd] : pk0[wd];
+        t[wd] = max_fields<BITS>(keep, __shfl_xor_sync(0xffffffffu, give, 1));
+    }
+    constexpr bool kTwo = kWords == 2;
+    const uint32_t keep = kTwo && below ? t[kWords - 1] : t[0], give = kTwo && !below ? t[kWords - 1] : t[0];
+    uint32_t w[1] = {max_fields<BITS>(keep, __shfl_xor_sync(0xffffffffu, give, 8))};
+    const bool strip1 = e.two && right;
+    const bool mine = (strip1 ? e.store[1] : e.store[0]) && (e.two || !right) && (kTwo || !below);
+    const int first = kTwo && below ? HB / 2 : 0;  // of the lane's word
+    uint8_t *const dst = (strip1 ? e.dst[1] : e.dst[0]) + (m0 + first) * BITS / 8;
+    if (mine) store_packed<BITS, HB / kWords>(w, valid - first, dst);
+}
 
 // Staircase of Eq. 4 on a raw sum: how many of the channel's sorted thresholds
 // do not exceed it.  INT-4: the quarter by three pivots (piv, the same for all
@@ -1174,8 +1183,12 @@ __device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile &e)
             pack_values<BITS, kG>(y0, *reinterpret_cast<uint32_t(*)[kGW]>(pk0 + g0 / kG * kGW));
             pack_values<BITS, kG>(y1, *reinterpret_cast<uint32_t(*)[kGW]>(pk1 + g0 / kG * kGW));
         }
-        store_words<BITS, HB, POOL>(pk0, e.store[0], valid, e.dst[0] + m0 * BITS / 8);
-        if (e.two) store_words<BITS, HB, POOL>(pk1, e.store[1], valid, e.dst[1] + m0 * BITS / 8);
+        if constexpr (POOL) {
+            store_pooled<BITS, HB>(pk0, pk1, e, m0, valid);
+        } else {
+            if (e.store[0]) store_packed<BITS, HB>(pk0, valid, e.dst[0] + m0 * BITS / 8);
+            if (e.store[1]) store_packed<BITS, HB>(pk1, valid, e.dst[1] + m0 * BITS / 8);
+        }
     }
 }
 
@@ -1305,8 +1318,8 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
         for (int s = 0; s < 2; ++s) {
             const int ox = g.ox0 + s * kCols + oxr;
             if constexpr (POOL) {
-                // pooled pixel (oy/2, ox/2) is the 2x2 window of lanes L, L^1, L^8, L^9; its top-left lane stores
-                store[s] = (row & 9) == 0 && (oy >> 1) < a.pool_oh && (ox >> 1) < a.pool_ow;
+                // pooled pixel (oy/2, ox/2) is the 2x2 window of lanes L, L^1, L^8, L^9 (store_pooled)
+                store[s] = (oy >> 1) < a.pool_oh && (ox >> 1) < a.pool_ow;
                 dst[s] = a.y + ((static_cast<long long>(g.img) * a.pool_oh + (oy >> 1)) * a.pool_ow + (ox >> 1)) *
                                    out_row_bytes;
             } else {
@@ -1425,7 +1438,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
             prepare_filters<BITS, NT, FOLD>(a, smem, misc, w_full);
         }
         if (warp == kMmaWarp) {
-            if (convolve) mma_role<NT, BITS != 8>(a, smem, a_full, a_empty, acc_full, acc_empty, done, misc);
+            if (convolve) mma_role<NT, BITS != 8, FOLD>(a, smem, a_full, a_empty, acc_full, acc_empty, done, misc);
         } else {
             // all slots start free (the MMA warp writes each accumulator's pre-load)
             if (convolve && (threadIdx.x & 31) == 0)

@@ -277,16 +277,28 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
         : "memory");
 }
 
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // Field-wise unsigned maximum of two words of packed Q-bit values (Q = 8, 4, 2).
+// INT-8: the larger halfword has the larger high byte; the low bytes by themselves.
 // INT-4: bit 3 of (a | 8) - (b & 7) says whether a's low three bits are not below
 // b's (no borrow leaves the field); with the top bits it gives a >= b, spread to
 // the field.  INT-2: the high bits' OR, and the low bit of whichever high bit is
-// not the smaller one.  8 and 7 operations; byte-wise maxima of the masked words
-// took about 40 and 80, and made INT-2 pooling compute-bound.
+// not the smaller one.  5, 8 and 7 operations; a byte-wise maximum (__vmaxu4) takes
+// about 20, which made the fused INT-8 pool the slowest part of its layers, and
+// INT-2 pooling (four of them on masked words) compute-bound.
 template <int BITS>
 __device__ __forceinline__ uint32_t max_fields(uint32_t a, uint32_t b)
 {
-    if (BITS == 8) return __vmaxu4(a, b);
+    if (BITS == 8) {
+        constexpr uint32_t kEven = 0x00FF00FFu;
+        return (max_u16x2(a, b) & ~kEven) | max_u16x2(a & kEven, b & kEven);
+    }
     if (BITS == 4) {
         constexpr uint32_t kTop = 0x88888888u;
         const uint32_t low = (a | kTop) - (b & ~kTop);
