@@ -122,7 +122,7 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
             return c;
         default: break;
     }
-    c.wplan = plan_conv_win(s);
+    c.wplan = plan_conv_win_batch(s);
     if (c.wplan.ok) {
         c.kernel = kWindow;
         return c;
@@ -134,7 +134,7 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
         c.kernel = general_or_wide(&c, s);
         if (c.kernel == kGeneral) {
             // one-shot calls: the window kernel on windows read as whole image rows
-            c.wplan = plan_conv_win(s, true);
+            c.wplan = plan_conv_win_batch(s, true);
             if (c.wplan.ok) c.kernel = kRows;
         }
     } else if (d->algo != QNN_ALGO_TENSORCORE) {
@@ -395,13 +395,13 @@ qnn_status qconv_hwc_pool2_run(const qnn_conv_desc *d, const void *x, void *y, c
     if (s.oh < 2 || s.ow < 2) return QNN_EINVAL;  // no pooled pixel
     if (s.n > 0 && (!x || !y)) return QNN_EINVAL;
     if (!aligned(x, 16) || !aligned(y, 16)) return QNN_EALIGN;
-    // the kernel and plan qconv_hwc_prepare chose for this descriptor (the window
-    // planner's layout does not depend on the fused pool)
+    // the kernel qconv_hwc_prepare chose for this descriptor, and a plan with the same
+    // prepared image (with the pool, stacked images take an even number of rows each)
+    s.pool = 1;
     const Choice c = choose(d, s);
     if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
     if (c.kernel != kWindow) return QNN_EUNSUPPORTED;
     if (!workspace || workspace_bytes < c.wplan.img_bytes || !aligned(workspace, 256)) return QNN_EWORKSPACE;
-    s.pool = 1;
     ConvParams p{};
     p.x = static_cast<const uint8_t *>(x);
     p.y = static_cast<uint8_t *>(y);
@@ -458,7 +458,7 @@ qnn_status qconv_hwc_binary(const qnn_conv_desc *d, const void *x, const void *w
     // 128 products per output on: below that the counts are few (209 images of 7 x 20 x 32 -> 88, 1 x 1: 6.8 us
     // with counts, 11.5 there; 299 of 30 x 28 x 64 -> 104, 1 x 1: 21.7 and 20.6; 3 x 3 layers of 32 channels 26.4 and 9.7)
     const bool many = static_cast<long long>(s.kh) * s.kw * s.c >= 128;
-    const WinPlan wplan = many ? plan_conv_win(s) : WinPlan{};
+    const WinPlan wplan = many ? plan_conv_win_batch(s) : WinPlan{};
     if (wplan.ok && wplan.nch_max == 1 && aligned(x, 16) && aligned(w, 16)) {
         ConvParams p{};
         p.x = static_cast<const uint8_t *>(x);

@@ -26,7 +26,7 @@ int strips_per_tile(int ow)
 
 }  // namespace
 
-WinPlan plan_conv_win(const ConvShape &s, bool rows)
+WinPlan plan_conv_win(const ConvShape &s, bool rows, int period)
 {
     WinPlan p{};
     p.ok = false;
@@ -77,7 +77,7 @@ WinPlan plan_conv_win(const ConvShape &s, bool rows)
             if (cb % 16 != 0) continue;  // per-row copies start at any pixel
             raw_row_bytes = round_up(static_cast<uint32_t>(std::min(sp, s.w) * cb), 16);
         }
-        const uint32_t raw_bytes = round_up(static_cast<uint32_t>(std::min(wh, s.h)) * raw_row_bytes, 128);
+        const uint32_t raw_bytes = round_up(static_cast<uint32_t>(period ? wh : std::min(wh, s.h)) * raw_row_bytes, 128);
         if (raw_bytes >= (1u << 20)) continue;  // one transaction count
         const uint32_t p_alloc = round_up(static_cast<uint32_t>(wh * sp), 8);
         const uint32_t chunk_stride = p_alloc * 16;
@@ -148,10 +148,13 @@ WinPlan plan_conv_win(const ConvShape &s, bool rows)
         p.wh = wh;
         p.p_alloc = static_cast<int>(p_alloc);
         p.tiles_x = tiles_x;
-        p.tiles_y = (s.oh + win::kRows - 1) / win::kRows;
-        p.tiles_per_img = p.tiles_x * p.tiles_y;
-        p.total_tiles = static_cast<long long>(s.n) * p.tiles_per_img;
-        if (p.total_tiles >= (1ll << 31)) return p;
+        p.period = period;
+        const long long rows_all = period ? (s.n - 1ll) * period + s.oh : s.oh;
+        const long long tiles_y = (rows_all + win::kRows - 1) / win::kRows;
+        p.total_tiles = (period ? 1 : s.n) * tiles_x * tiles_y;
+        if (p.total_tiles >= (1ll << 31) || (period && rows_all >= (1ll << 30))) return p;
+        p.tiles_y = static_cast<int>(tiles_y);
+        p.tiles_per_img = static_cast<int>(tiles_x * tiles_y);
         p.full_rows = full_rows;
         p.raw_row_bytes = raw_row_bytes;
         p.raw_bytes = raw_bytes;
@@ -165,6 +168,22 @@ WinPlan plan_conv_win(const ConvShape &s, bool rows)
         return p;
     }
     return p;
+}
+
+WinPlan plan_conv_win_batch(const ConvShape &s, bool rows)
+{
+    const WinPlan p = plan_conv_win(s, rows);
+    if (!p.ok || s.n < 2) return p;
+    // rows per image: the image and one padding, an even count for the pool's windows
+    int period = s.h + s.ph;
+    if (s.pool) period += period & 1;
+    // (an image's outputs have to fit its rows, and the kernel divides rows of a window in 32 bits)
+    if (s.oh > period || period < 2 || period > 4096) return p;
+    const long long rows_all = (s.n - 1ll) * period + s.oh, tiles = (rows_all + win::kRows - 1) / win::kRows * p.tiles_x;
+    const long long sms = device_sm_count();
+    if ((tiles + sms - 1) / sms >= (p.total_tiles + sms - 1) / sms) return p;
+    const WinPlan q = plan_conv_win(s, rows, period);
+    return q.ok && q.s == p.s && q.a_stages == p.a_stages ? q : p;
 }
 
 namespace {
@@ -201,6 +220,10 @@ win::WinArgs win_args(const WinPlan &plan, const ConvShape &s, const ConvParams 
     a.fd_tpi = make_fastdiv(static_cast<uint32_t>(plan.tiles_per_img));
     a.fd_tx = make_fastdiv(static_cast<uint32_t>(plan.tiles_x));
     a.fd_sp = make_fastdiv(static_cast<uint32_t>(plan.sp));
+    a.per = plan.period ? plan.period : INT32_MAX;
+    a.fd_per = make_fastdiv(static_cast<uint32_t>(a.per));
+    // ceil(2^32 / period): exact for rows below 2^32 / period (at most 4096 + 23 of them)
+    a.m_per = plan.period ? static_cast<uint32_t>(((1ull << 32) + plan.period - 1) / plan.period) : 0u;
     a.raw_stages = plan.raw_stages;
     a.a_stages = plan.a_stages;
     a.nch_max = plan.nch_max;

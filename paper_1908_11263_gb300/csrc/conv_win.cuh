@@ -18,6 +18,11 @@
 // 8-row core-matrix groups are the sixteen output rows, sp positions apart.
 // One shared-memory descriptor per MMA, no im2col buffer and no shifted
 // copies (Eq. 7: neighbouring output pixels read neighbouring window pixels).
+// Images whose height fills the last tile badly are stacked: the batch is one tall
+// image in which pad_h zero rows stand between two images (above the next one
+// and below the last: what lies past an image's end is the next one's padding),
+// and tiles run across them.  56 x 56 rows take 57 rows per image instead of 64,
+// 8 x 8 ones with pad 2 take 10 instead of 16.
 // With few input channels (INT-8, c * kw <= 16) the kernel columns fold into
 // K instead: a staged position holds the c channels of kw neighbouring pixels,
 // the window is 8S positions wide and each MMA covers one kernel row.
@@ -130,6 +135,11 @@ struct WinArgs {
     int full_rows;
     int tiles_x, tiles_per_img, total_tiles;
     FastDiv fd_tpi, fd_tx, fd_sp;
+    // Stacked images (WinPlan::period): rows per image, and the reciprocals of that count for any row of
+    // the batch and (32 bits) for a row of a window.  Not stacked: a count above every row, reciprocal 0.
+    int per;
+    FastDiv fd_per;
+    uint32_t m_per;
     int raw_stages, a_stages, nch_max, nch_min;
     uint32_t raw_row_bytes, raw_bytes, chunk_stride, stage_bytes;
     uint32_t off_b, off_a, off_raw, off_rec, off_thr, off_tap, off_bar;
@@ -147,30 +157,55 @@ struct WinArgs {
     int *status;
 };
 
-// Tile t: image, first output row and column, window origin in the input.
+// Tile t: image, first output row and column, window origin in the input.  Stacked
+// images: the image that the tile's first row belongs to, and the row within
+// that image's period; the tile's further rows may belong to the next images.
 struct Geo {
-    int img, oy0, ox0, iy0, ix0;
+    int img, oy0, ox0, ix0;
 };
 
+template <bool STACK>
 __device__ __forceinline__ Geo geo_of(const WinArgs &a, int t)
 {
     Geo g;
     g.img = fdiv(t, a.fd_tpi);
     const int ti = t - g.img * a.tiles_per_img;
     const int ty = fdiv(ti, a.fd_tx);
-    g.oy0 = ty * kRows;
+    const int q = STACK ? fdiv(ty * kRows, a.fd_per) : 0;
+    g.img += q;
+    g.oy0 = ty * kRows - q * a.per;
     g.ox0 = (ti - ty * a.tiles_x) * (kCols * a.s);
-    g.iy0 = g.oy0 - a.ph;
     g.ix0 = g.ox0 - a.pw;
     return g;
 }
 
-// Window rows [r_lo, r_hi) and columns [c_lo, c_hi) that lie inside the image.
-__device__ __forceinline__ int row_lo(const WinArgs &a, const Geo &g) { return min(a.wh, max(0, -g.iy0)); }
-__device__ __forceinline__ int row_hi(const WinArgs &a, const Geo &g)
+// Row `oy0 + r` of the tile (r below the window's height): images past g.img, and
+// the row within that image's period.
+struct TileRow {
+    int q, row;
+};
+
+template <bool STACK>
+__device__ __forceinline__ TileRow tile_row(const WinArgs &a, const Geo &g, int r)
 {
-    return max(row_lo(a, g), min(a.wh, a.h - g.iy0));
+    const int y = g.oy0 + r;
+    if (!STACK) return {0, y};
+    const int q = static_cast<int>(__umulhi(static_cast<uint32_t>(y), a.m_per));
+    return {q, y - q * a.per};
 }
+
+// Input rows of image g.img and those after it that stand before row r of the
+// tile's window.  The rows a window holds are consecutive in the input, also
+// across images: [rows_before(0), rows_before(wh)).
+template <bool STACK>
+__device__ __forceinline__ int rows_before(const WinArgs &a, const Geo &g, int r)
+{
+    const TileRow t = tile_row<STACK>(a, g, r);
+    if (STACK && t.q >= a.n - g.img) return (a.n - g.img) * a.h;
+    return t.q * a.h + min(a.h, max(0, t.row - a.ph));
+}
+
+// Window columns [c_lo, c_hi) that lie inside the image.
 __device__ __forceinline__ int col_lo(const WinArgs &a, const Geo &g) { return min(a.sp, max(0, -g.ix0)); }
 __device__ __forceinline__ int col_hi(const WinArgs &a, const Geo &g)
 {
@@ -199,25 +234,26 @@ __device__ __forceinline__ void load_filters(const WinArgs &a, uint8_t *smem, ui
 // The input rows of up to `count` more tiles' windows: one bulk copy when
 // windows span whole image rows, else one per row (lanes issue them in
 // parallel).
+template <bool STACK>
 __device__ __forceinline__ void load_windows(const WinArgs &a, uint8_t *smem, uint64_t *raw_full, uint64_t *raw_empty,
                                              LoadState &st, int count)
 {
     const int lane = threadIdx.x & 31;
     for (; st.t < a.total_tiles && count > 0; st.t += gridDim.x, --count) {
-        const Geo g = geo_of(a, st.t);
-        const int r0 = row_lo(a, g), r1 = row_hi(a, g);
+        const Geo g = geo_of<STACK>(a, st.t);
+        const int b0 = rows_before<STACK>(a, g, 0), rows = rows_before<STACK>(a, g, a.wh) - b0;
+        const long long row0 = static_cast<long long>(g.img) * a.h + b0;
         const int c0 = col_lo(a, g), c1 = col_hi(a, g);
         if (!mbar_wait_warp(&raw_empty[st.rs], st.ph ^ 1u, a.status)) {
             st.t = a.total_tiles;  // give up: the other roles time out as well
             break;
         }
         uint8_t *dst = smem + a.off_raw + st.rs * a.raw_bytes;
-        const int rows = r1 - r0;
         if (a.full_rows) {
             const uint32_t bytes = static_cast<uint32_t>(rows) * a.raw_row_bytes;
             if (lane == 0) {
                 mbar_arrive_expect_tx(&raw_full[st.rs], bytes);
-                const uint8_t *src = a.x + (static_cast<long long>(g.img) * a.h + (g.iy0 + r0)) * a.raw_row_bytes;
+                const uint8_t *src = a.x + row0 * a.raw_row_bytes;
                 for (uint32_t off = 0; off < bytes; off += 32768u)
                     bulk_g2s(dst + off, src + off, min(32768u, bytes - off), &raw_full[st.rs]);
             }
@@ -226,11 +262,9 @@ __device__ __forceinline__ void load_windows(const WinArgs &a, uint8_t *smem, ui
             if (lane == 0) mbar_arrive_expect_tx(&raw_full[st.rs], seg * static_cast<uint32_t>(rows));
             __syncwarp();
             if (seg)
-                for (int r = r0 + lane; r < r1; r += 32) {
-                    const uint8_t *src =
-                        a.x + ((static_cast<long long>(g.img) * a.h + (g.iy0 + r)) * a.w_ + (g.ix0 + c0)) * a.cb;
-                    bulk_g2s(dst + (r - r0) * a.raw_row_bytes, src, seg, &raw_full[st.rs]);
-                }
+                for (int r = lane; r < rows; r += 32)
+                    bulk_g2s(dst + r * a.raw_row_bytes, a.x + ((row0 + r) * a.w_ + (g.ix0 + c0)) * a.cb, seg,
+                             &raw_full[st.rs]);
         }
         __syncwarp();
         ++st.issued;
@@ -283,7 +317,7 @@ __device__ __forceinline__ uint4 stage_chunk(uint2 v)
 // packed channels (16-byte loads when a pixel is a whole number of 16-byte
 // units, else 8-byte ones) and stores one 16-byte chunk per K-chunk plane, so
 // a warp's stores are consecutive positions of a plane.
-template <int BITS>
+template <int BITS, bool STACK>
 __device__ __forceinline__ void converter_role(const WinArgs &a, uint8_t *smem, uint64_t *raw_full, uint64_t *raw_empty,
                                                uint64_t *a_full, uint64_t *a_empty)
 {
@@ -297,8 +331,8 @@ __device__ __forceinline__ void converter_role(const WinArgs &a, uint8_t *smem, 
     int rs = 0, as = 0;
     uint32_t r_ph = 0, a_ph = 0;
     for (int t = blockIdx.x; t < a.total_tiles; t += gridDim.x) {
-        const Geo g = geo_of(a, t);
-        const int r0 = row_lo(a, g), r1 = row_hi(a, g);
+        const Geo g = geo_of<STACK>(a, t);
+        const int b0 = rows_before<STACK>(a, g, 0), images = a.n - g.img;
         const int c0 = col_lo(a, g), c1 = col_hi(a, g);
         // raw column of window column px: the copied span starts at window column c0
         // (whole rows start at image column 0, i.e. window column -ix0)
@@ -319,9 +353,12 @@ __device__ __forceinline__ void converter_role(const WinArgs &a, uint8_t *smem, 
             for (int u = 0; u < 3; ++u) {
                 const int pos = pos0 + u * 128;
                 const int pr = fdiv(pos, a.fd_sp), pc = pos - pr * a.sp;
-                ok[u] = pos < a.npos && pr >= r0 && pr < r1 && pc >= c0 && pc < c1;
+                const TileRow tr = tile_row<STACK>(a, g, pr);
+                const int iy = tr.row - a.ph;
+                ok[u] = pos < a.npos && static_cast<unsigned>(iy) < static_cast<unsigned>(a.h) && (!STACK || tr.q < images) &&
+                        pc >= c0 && pc < c1;
                 // the pixel's packed channels (a safe address where the value is padding)
-                const uint8_t *q = raw + (ok[u] ? static_cast<uint32_t>(pr - r0) * a.raw_row_bytes +
+                const uint8_t *q = raw + (ok[u] ? static_cast<uint32_t>(tr.q * a.h + iy - b0) * a.raw_row_bytes +
                                                       static_cast<uint32_t>((pc + base_col) * a.cb)
                                                 : 0u);
                 if (BITS == 1) {  // at most four words
@@ -384,6 +421,7 @@ __device__ __forceinline__ void converter_role(const WinArgs &a, uint8_t *smem, 
 // raw stage holds whole image rows.  Activation 0 stands outside the image
 // (it stages as -128, like every padded value); the values past kw * c meet
 // zero weights.
+template <bool STACK>
 __device__ __forceinline__ void converter_fold(const WinArgs &a, uint8_t *smem, uint64_t *raw_full,
                                                uint64_t *raw_empty, uint64_t *a_full, uint64_t *a_empty)
 {
@@ -391,8 +429,8 @@ __device__ __forceinline__ void converter_fold(const WinArgs &a, uint8_t *smem, 
     int rs = 0, as = 0;
     uint32_t r_ph = 0, a_ph = 0;
     for (int t = blockIdx.x; t < a.total_tiles; t += gridDim.x) {
-        const Geo g = geo_of(a, t);
-        const int r0 = row_lo(a, g), r1 = row_hi(a, g);
+        const Geo g = geo_of<STACK>(a, t);
+        const int b0 = rows_before<STACK>(a, g, 0), images = a.n - g.img;
         if (!mbar_wait_warp(&raw_full[rs], r_ph, a.status)) return;
         if (!mbar_wait_warp(&a_empty[as], a_ph ^ 1u, a.status)) return;
         const uint8_t *raw = smem + a.off_raw + rs * a.raw_bytes;
@@ -404,8 +442,10 @@ __device__ __forceinline__ void converter_fold(const WinArgs &a, uint8_t *smem, 
             // the span's pixels inside the image, [jlo, jhi); their bytes are contiguous in the row
             const int jlo = max(0, -col), jhi = min(a.kw, a.w_ - col);
             unsigned long long lo = 0ull, hi = 0ull;  // the 16 bytes, zero outside the image
-            if (pr >= r0 && pr < r1 && jhi > jlo) {
-                const uint8_t *row = raw + static_cast<uint32_t>(pr - r0) * a.raw_row_bytes;
+            const TileRow tr = tile_row<STACK>(a, g, pr);
+            const int iy = tr.row - a.ph;
+            if (static_cast<unsigned>(iy) < static_cast<unsigned>(a.h) && (!STACK || tr.q < images) && jhi > jlo) {
+                const uint8_t *row = raw + static_cast<uint32_t>(tr.q * a.h + iy - b0) * a.raw_row_bytes;
                 // five aligned words from the first inside byte, funnel-shifted to it
                 const uint32_t off = static_cast<uint32_t>((col + jlo) * a.c);
                 const uint32_t *wp = reinterpret_cast<const uint32_t *>(row + (off & ~3u));
@@ -1244,7 +1284,7 @@ __device__ __forceinline__ void epi_binary(const WinArgs &a, const EpiTile &e, b
     }
 }
 
-template <int BITS, int NT, bool POOL>
+template <int BITS, int NT, bool POOL, bool STACK>
 __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, uint64_t *acc_full, uint64_t *acc_empty,
                                               const Misc *misc)
 {
@@ -1307,10 +1347,12 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
     const int oyr = row >> 3, oxr = row & 7;
     for (int i = 0, t = blockIdx.x; t < a.total_tiles; ++i, t += gridDim.x) {
         const int slot = i % nslots;
-        const Geo g = geo_of(a, t);
+        const Geo g = geo_of<STACK>(a, t);
         if (!mbar_wait_warp(&acc_full[slot], (i / nslots) & 1, status)) return;
         tc_fence_after();
-        const int oy = g.oy0 + oyr;
+        const TileRow tr = tile_row<STACK>(a, g, oyr);
+        const int oy = tr.row, img = g.img + tr.q;
+        const bool real = !STACK || tr.q < a.n - g.img;
         // where strip s's pixel of this lane goes: its output row, or its pooled pixel
         uint8_t *dst[2];
         bool store[2];
@@ -1319,12 +1361,12 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
             const int ox = g.ox0 + s * kCols + oxr;
             if constexpr (POOL) {
                 // pooled pixel (oy/2, ox/2) is the 2x2 window of lanes L, L^1, L^8, L^9 (store_pooled)
-                store[s] = (oy >> 1) < a.pool_oh && (ox >> 1) < a.pool_ow;
-                dst[s] = a.y + ((static_cast<long long>(g.img) * a.pool_oh + (oy >> 1)) * a.pool_ow + (ox >> 1)) *
+                store[s] = real && (oy >> 1) < a.pool_oh && (ox >> 1) < a.pool_ow;
+                dst[s] = a.y + ((static_cast<long long>(img) * a.pool_oh + (oy >> 1)) * a.pool_ow + (ox >> 1)) *
                                    out_row_bytes;
             } else {
-                store[s] = oy < a.oh && ox < a.ow;
-                dst[s] = a.y + ((static_cast<long long>(g.img) * a.oh + oy) * a.ow + ox) * out_row_bytes;
+                store[s] = real && oy < a.oh && ox < a.ow;
+                dst[s] = a.y + ((static_cast<long long>(img) * a.oh + oy) * a.ow + ox) * out_row_bytes;
             }
             store[s] = store[s] && (s == 0 || two);
         }
@@ -1361,7 +1403,7 @@ __device__ __forceinline__ void epilogue_role(const WinArgs &a, uint8_t *smem, u
 
 // ---------------------------------------------------------------- the kernel
 
-template <int BITS, int NT, bool POOL, bool FOLD>
+template <int BITS, int NT, bool POOL, bool FOLD, bool STACK>
 __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
 {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -1421,14 +1463,14 @@ __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
     const bool convolve = a.img_out == nullptr;
     if (warp < kConvWarps) {
         if (convolve) {
-            if constexpr (BITS == 8 && FOLD) converter_fold(a, smem, raw_full, raw_empty, a_full, a_empty);
-            else converter_role<BITS>(a, smem, raw_full, raw_empty, a_full, a_empty);
+            if constexpr (BITS == 8 && FOLD) converter_fold<STACK>(a, smem, raw_full, raw_empty, a_full, a_empty);
+            else converter_role<BITS, STACK>(a, smem, raw_full, raw_empty, a_full, a_empty);
         }
     } else if (warp == kLoadWarp) {
         if (!a.img) load_filters(a, smem, w_full);
         if (convolve) {
             LoadState ld{0, 0, static_cast<int>(blockIdx.x), 0u};
-            load_windows(a, smem, raw_full, raw_empty, ld, a.total_tiles);
+            load_windows<STACK>(a, smem, raw_full, raw_empty, ld, a.total_tiles);
             load_drain(a, raw_full, w_full, ld);
         }
     } else {
@@ -1444,7 +1486,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
             if (convolve && (threadIdx.x & 31) == 0)
                 for (uint32_t slot = 0; slot < misc->nslots; ++slot) mbar_arrive(&acc_empty[slot]);
             if (!a.img) prepare_records<BITS, NT>(a, smem, misc);
-            if (convolve) epilogue_role<BITS, NT, POOL>(a, smem, acc_full, acc_empty, misc);
+            if (convolve) epilogue_role<BITS, NT, POOL, STACK>(a, smem, acc_full, acc_empty, misc);
         }
         if (!convolve) {
             prep_sync();

@@ -14,13 +14,13 @@
 namespace qnn {
 namespace {
 
-template <int BITS, int NT, bool POOL, bool FOLD = false>
-cudaError_t launch_one(const win::WinArgs &a, int grid, uint32_t smem, cudaStream_t st)
+template <int BITS, int NT, bool POOL, bool FOLD, bool STACK>
+cudaError_t launch_kern(const win::WinArgs &a, int grid, uint32_t smem, cudaStream_t st)
 {
     // the opt-in shared-memory limit is raised once per device, outside any stream capture
     static std::mutex mu;
     static bool raised[64] = {};
-    auto kern = win::conv_win_kernel<BITS, NT, POOL, FOLD>;
+    auto kern = win::conv_win_kernel<BITS, NT, POOL, FOLD, STACK>;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -46,6 +46,15 @@ cudaError_t launch_one(const win::WinArgs &a, int grid, uint32_t smem, cudaStrea
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// Stacked images have their own instantiations: with the rows' divisions in the
+// plain kernel the benchmark layer took 12.2 us instead of 11.2.
+template <int BITS, int NT, bool POOL, bool FOLD = false>
+cudaError_t launch_one(const win::WinArgs &a, int grid, uint32_t smem, cudaStream_t st)
+{
+    return a.m_per ? launch_kern<BITS, NT, POOL, FOLD, true>(a, grid, smem, st)
+                   : launch_kern<BITS, NT, POOL, FOLD, false>(a, grid, smem, st);
 }
 
 }  // namespace
