@@ -1061,9 +1061,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_gather_kernel(const Args a)
     extern __shared__ __align__(128) uint8_t smem[];
     Shared *sh = reinterpret_cast<Shared *>(smem + a.off_bar);
     const int warp = threadIdx.x >> 5;
-    // the next kernel in the stream may launch now; it waits for this one
-    // before it touches memory
-    pdl_trigger();
     if (warp == kMmaWarp) {
         if ((threadIdx.x & 31) == 0) {
             // pixel stages: four warps each (im2col), all eight (flat window; converted filters behind the pixels)
@@ -1099,8 +1096,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_gather_kernel(const Args a)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem;
-    // everything the previous kernel in the stream wrote is visible from here on
+    // everything the previous kernel in the stream wrote is visible from here on, and
+    // the next kernel may launch; it waits for this one before it touches memory
     pdl_wait();
+    pdl_trigger();
 
     // the grid is a multiple of the channel blocks: a CTA keeps one block
     const int nt = static_cast<int>(blockIdx.x) % a.n_ntiles, mt0 = static_cast<int>(blockIdx.x) / a.n_ntiles;

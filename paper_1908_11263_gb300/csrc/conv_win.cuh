@@ -1418,13 +1418,6 @@ __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
     uint64_t *w_full = done + 1;
     Misc *misc = reinterpret_cast<Misc *>(w_full + 2);  // (one spare barrier slot)
     const int warp = threadIdx.x >> 5;
-    // Programmatic dependent launch: the next kernel in the stream may launch
-    // now; its blocks take each SM as this kernel's block there exits, and do
-    // their setup while the rest of this grid finishes.  A launch that writes
-    // a prepared image (img_out) does not: its successor starts after it ends,
-    // so a convolving launch may read its image before waiting on its
-    // predecessor (every image was written by an earlier, finished launch).
-    if (a.img_out == nullptr) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == kMmaWarp) {
         if ((threadIdx.x & 31) == 0) {
@@ -1449,11 +1442,18 @@ __global__ void __launch_bounds__(kThreads, 1) conv_win_kernel(const WinArgs a)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // the prepared image comes from a finished launch: its copy may start now
+    // The prepared image comes from a launch that has ended, so its copy may start
+    // now: the launch just before this one has passed its own wait (no kernel
+    // releases its successor earlier), hence all before it have ended, and it is not
+    // the one that wrote the image (a preparing launch releases no successor).
     if (warp == kLoadWarp && a.img) load_image(a, smem, w_full);
     // nothing above reads other global memory: from here on, everything the
     // previous kernel in the stream wrote is visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    // Programmatic dependent launch: the next kernel in the stream may launch
+    // now; its blocks take each SM as this kernel's block there exits, and do
+    // their setup while the rest of this grid finishes.
+    if (a.img_out == nullptr) pdl_trigger();
 
     // Each warp takes its role.  The loader copies the filters (or the
     // prepared image), then streams the windows; the converters stage windows

@@ -20,12 +20,17 @@ __device__ __forceinline__ void report(int *status, int code) { atomicCAS(status
 // Programmatic dependent launch: a primary grid lets the next kernel of the
 // stream start early (pdl_trigger); that kernel calls pdl_wait before it
 // touches the primary's results.  Both are no-ops without such a launch.
+// A kernel launched that way releases its successor only after its own wait:
+// whatever runs ahead of its wait then knows every launch but its direct
+// predecessor to have ended, which is what a prepared image read that early
+// relies on (with the release ahead of the wait a chain of short launches let
+// the image be read while a launch two before was still writing).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Launch with programmatic stream serialization: the kernel may start while
-// its predecessor in the stream still runs, and calls pdl_wait before it
-// touches global memory.
+// its predecessor in the stream still runs, and calls pdl_wait, then
+// pdl_trigger, before it touches global memory.
 template <class... Params, class... Args>
 cudaError_t launch_pdl(void (*kern)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
                        Args... args)

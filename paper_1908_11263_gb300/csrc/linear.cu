@@ -71,8 +71,8 @@ constexpr int kSmemRowsMax = 200 * 1024;  // weight bytes kept in shared memory
 __global__ void __launch_bounds__(256) linear_smem_kernel(int n, int k, int m, const uint8_t *x, const int8_t *w,
                                                           const int32_t *bias, int32_t *y)
 {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     extern __shared__ uint4 wsh[];  // [m][k/16]
     const int kv = k / 16;
     const uint4 *wg = reinterpret_cast<const uint4 *>(w);

@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(kThreads) pack_kernel(const int8_t *src, uint8
                                                         long long nbytes)
 {
     using P = typename PackedGroup<BITS>::type;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const long long g0 = static_cast<long long>(blockIdx.x) * (kThreads * kGroups) + threadIdx.x;
     uint4 v[kGroups];
 #pragma unroll
@@ -139,8 +139,8 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const uint8_t *src, in
                                                           long long nbytes, int is_signed)
 {
     using P = typename PackedGroup<BITS>::type;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const long long g0 = static_cast<long long>(blockIdx.x) * (kThreads * kGroups) + threadIdx.x;
     P v[kGroups];
 #pragma unroll

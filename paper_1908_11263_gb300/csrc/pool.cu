@@ -21,8 +21,8 @@ __global__ void __launch_bounds__(256) maxpool_vec_kernel(unsigned total, int h,
                                                           FastDiv fd_vec, FastDiv fd_ow, FastDiv fd_oh, const uint4 *x,
                                                           uint4 *y)
 {
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();
     const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= total) return;
     const int pix = fdiv(static_cast<int>(gid), fd_vec), v = static_cast<int>(gid) - pix * vec_per_pix;
