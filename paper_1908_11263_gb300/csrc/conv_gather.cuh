@@ -175,7 +175,7 @@ struct Gran<false> {
         if (hi > lo && a >= begin && a + 20 <= end) {
             const uint32_t *q4 = reinterpret_cast<const uint32_t *>(a);
 #pragma unroll
-            for (int k = 0; k < 5; ++k) q[k] = __ldg(q4 + k);
+            for (int k = 0; k < 5; ++k) q[k] = q4[k];
             return;
         }
         const int b0 = lo + static_cast<int>(sh), b1 = hi + static_cast<int>(sh);
@@ -184,7 +184,7 @@ struct Gran<false> {
         if (hi > lo) {
 #pragma unroll
             for (int b = 0; b < 20; ++b)
-                if (b >= b0 && b < b1) q[b / 4] |= static_cast<uint32_t>(__ldg(a + b)) << (8 * (b % 4));
+                if (b >= b0 && b < b1) q[b / 4] |= static_cast<uint32_t>(a[b]) << (8 * (b % 4));
         }
     }
     __device__ __forceinline__ uint4 get() const
@@ -227,7 +227,7 @@ __device__ __forceinline__ void fetch_w(const Args &a, int o, int g, Gran<ALIGNE
     }
     const int i = fdiv(g, a.fd_gr), r = (g - i * static_cast<int>(a.fd_gr.d)) * 16;
     const uint8_t *p = a.w + static_cast<uint32_t>((o * a.kh + i) * a.kwc + r);
-    if constexpr (ALIGNED) v.v = __ldg(reinterpret_cast<const uint4 *>(p));
+    if constexpr (ALIGNED) v.v = *reinterpret_cast<const uint4 *>(p);
     else v.load(p, 0, min(16, a.kwc - r), a.w, a.w + a.wbytes);
 }
 
@@ -396,7 +396,7 @@ __device__ __forceinline__ void fetch_x(const Args &a, const Shared *sh, const P
             const bool ok = in && static_cast<unsigned>(px.iy[it] + i) < static_cast<unsigned>(a.h) &&
                             static_cast<unsigned>(px.ix[it] + j) < static_cast<unsigned>(a.w_);
             v[it].zero();
-            if (ok) v[it].v = __ldg(reinterpret_cast<const uint4 *>(a.x + (px.base[it] + off)));
+            if (ok) v[it].v = *reinterpret_cast<const uint4 *>(a.x + (px.base[it] + off));
         }
     } else {
 #pragma unroll
@@ -499,7 +499,7 @@ __device__ __forceinline__ void produce_flat(const Args &a, uint8_t *smem, Share
         for (int it = 0; it < kMaxIter; ++it) {
             v[it] = make_uint4(0, 0, 0, 0);
             if (base[it] != kOutside && g < a.cgr)
-                v[it] = __ldg(reinterpret_cast<const uint4 *>(a.x + (base[it] + static_cast<uint32_t>(g) * 16u)));
+                v[it] = *reinterpret_cast<const uint4 *>(a.x + (base[it] + static_cast<uint32_t>(g) * 16u));
         }
     };
     if (mt0 >= a.mtiles) return;
@@ -624,7 +624,7 @@ __device__ __forceinline__ Chunks make_chunks(const Args &a, Shared *sh, int nt)
         const int o = nt * a.w_rows + (et & (kRowsW - 1));
         if (et < kEpiWarps * 32 && (et & (kRowsW - 1)) < a.w_rows)
             for (int s = et / kRowsW; s < a.nxs; s += kEpiWarps * 32 / kRowsW)
-                atomicMax(&sh->abs_max[s], __ldg(a.wabs + static_cast<size_t>(o) * kMaxAbs + s));
+                atomicMax(&sh->abs_max[s], a.wabs[static_cast<size_t>(o) * kMaxAbs + s]);
         chunk_sync();
         c.every = 0;
         c.n = 1;

@@ -737,13 +737,13 @@ __device__ __forceinline__ void prepare_filters(const WinArgs &a, uint8_t *smem,
                     raw[b][gq] = make_uint2(lo, hi);
                 } else if (kGroupBytes == 8) {
                     const uint2 *q = reinterpret_cast<const uint2 *>(src + gq * 8);
-                    raw[b][gq] = !has ? make_uint2(0u, 0u) : copied ? *q : __ldg(q);
+                    raw[b][gq] = !has ? make_uint2(0u, 0u) : copied ? *q : ld_global(q);
                 } else if (kGroupBytes == 2) {
                     const uint16_t *q = reinterpret_cast<const uint16_t *>(src + gq * 2);
-                    raw[b][gq] = make_uint2(!has ? 0u : copied ? *q : __ldg(q), 0u);
+                    raw[b][gq] = make_uint2(!has ? 0u : copied ? *q : ld_global(q), 0u);
                 } else {
                     const uint32_t *q = reinterpret_cast<const uint32_t *>(src + gq * 4);
-                    raw[b][gq] = make_uint2(!has ? 0u : copied ? *q : __ldg(q), 0u);
+                    raw[b][gq] = make_uint2(!has ? 0u : copied ? *q : ld_global(q), 0u);
                 }
             }
         }

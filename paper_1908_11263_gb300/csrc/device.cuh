@@ -25,8 +25,33 @@ __device__ __forceinline__ void report(int *status, int code) { atomicCAS(status
 // predecessor to have ended, which is what a prepared image read that early
 // relies on (with the release ahead of the wait a chain of short launches let
 // the image be read while a launch two before was still writing).
+// Nor does such a kernel use __ldg: that load is for data nobody writes while
+// the kernel lives, and the direct predecessor may be writing its inputs then.
+// It reads them with ld_global, or plainly.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Coherent loads from global memory, kept behind pdl_wait and in their order.
+// (The window kernel's filters: with one generic load for both of their places the
+// 56 x 56 x 64 layer at batch 256 took 68.3 us instead of 66.5.)
+__device__ __forceinline__ uint2 ld_global(const uint2 *p)
+{
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint16_t *p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
 
 // Launch with programmatic stream serialization: the kernel may start while
 // its predecessor in the stream still runs, and calls pdl_wait, then

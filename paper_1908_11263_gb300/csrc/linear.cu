@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) linear_smem_kernel(int n, int k, int m, c
     extern __shared__ uint4 wsh[];  // [m][k/16]
     const int kv = k / 16;
     const uint4 *wg = reinterpret_cast<const uint4 *>(w);
-    for (int i = threadIdx.x; i < m * kv; i += blockDim.x) wsh[i] = __ldg(wg + i);
+    for (int i = threadIdx.x; i < m * kv; i += blockDim.x) wsh[i] = wg[i];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) linear_smem_kernel(int n, int k, int m, c
 #pragma unroll
             for (int j = 0; j < kOutChunk; ++j) acc[j] = 0;
             for (int i = lane; i < kv; i += 32) {
-                const uint4 xv = __ldg(xr + i);
+                const uint4 xv = xr[i];
 #pragma unroll
                 for (int j = 0; j < kOutChunk; ++j) {
                     if (o0 + j < m) {

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kThreads) pack_kernel(const int8_t *src, uint8
     uint4 v[kGroups];
 #pragma unroll
     for (int k = 0; k < kGroups; ++k)
-        if (g0 + k * kThreads < groups) v[k] = __ldg(reinterpret_cast<const uint4 *>(src) + g0 + k * kThreads);
+        if (g0 + k * kThreads < groups) v[k] = reinterpret_cast<const uint4 *>(src)[g0 + k * kThreads];
 #pragma unroll
     for (int k = 0; k < kGroups; ++k)
         if (g0 + k * kThreads < groups)
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads) unpack_kernel(const uint8_t *src, in
     P v[kGroups];
 #pragma unroll
     for (int k = 0; k < kGroups; ++k)
-        if (g0 + k * kThreads < groups) v[k] = __ldg(reinterpret_cast<const P *>(src) + g0 + k * kThreads);
+        if (g0 + k * kThreads < groups) v[k] = reinterpret_cast<const P *>(src)[g0 + k * kThreads];
 #pragma unroll
     for (int k = 0; k < kGroups; ++k)
         if (g0 + k * kThreads < groups) reinterpret_cast<uint4 *>(dst)[g0 + k * kThreads] = unpack16(v[k], is_signed != 0);

@@ -38,14 +38,14 @@ __global__ void __launch_bounds__(256) maxpool_vec_kernel(unsigned total, int h,
     };
     if (TWO) {
         const uint4 *low = src + static_cast<long long>(w) * vec_per_pix;
-        const uint4 t0 = __ldg(src), t1 = __ldg(src + vec_per_pix), t2 = __ldg(low), t3 = __ldg(low + vec_per_pix);
+        const uint4 t0 = src[0], t1 = src[vec_per_pix], t2 = low[0], t3 = low[vec_per_pix];
         take(t0);
         take(t1);
         take(t2);
         take(t3);
     } else {
         for (int i = 0; i < k; ++i)
-            for (int j = 0; j < k; ++j) take(__ldg(src + (static_cast<long long>(i) * w + j) * vec_per_pix));
+            for (int j = 0; j < k; ++j) take(src[(static_cast<long long>(i) * w + j) * vec_per_pix]);
     }
     y[gid] = best;
 }

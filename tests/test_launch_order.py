@@ -2,7 +2,8 @@
 
 A kernel that runs ahead of its own griddepcontrol.wait (the window kernel copies its prepared image there)
 relies on every launch but its direct predecessor having ended.  That holds when no kernel launched with
-programmatic serialization releases its successor before its own wait."""
+programmatic serialization releases its successor before its own wait.  And its inputs may still be written
+while it lives, which the read-only loads (__ldg) do not allow."""
 import glob
 import os
 import re
@@ -52,3 +53,22 @@ def test_successors_are_released_after_the_own_wait(name):
     wait = WAIT.search(body)
     assert wait is not None
     assert all(m.start() > wait.end() for m in TRIGGER.finditer(body))
+
+
+def overlapped_sources():
+    """(file, text without the kernels launched in full stream order) of the files with overlapped kernels."""
+    for path in sorted(glob.glob(os.path.join(qbuild.CSRC, "*.cu*"))):
+        with open(path) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        if os.path.basename(path) == "device.cuh" or not WAIT.search(text):
+            continue
+        for name, (_, body) in KERNELS.items():
+            if name in PLAIN or not WAIT.search(body):
+                text = text.replace(body, "")
+        yield os.path.basename(path), text
+
+
+def test_no_read_only_loads_where_the_predecessor_may_still_write():
+    texts = dict(overlapped_sources())
+    assert {"pack.cu", "pool.cu", "linear.cu", "conv_win.cuh", "conv_gather.cuh"} <= set(texts)
+    assert [name for name, text in texts.items() if re.search(r"__ldg|ld\.global\.nc|__restrict__", text)] == []
