@@ -1096,10 +1096,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_gather_kernel(const Args a)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem;
-    // everything the previous kernel in the stream wrote is visible from here on, and
-    // the next kernel may launch; it waits for this one before it touches memory
+    // everything the previous kernel in the stream wrote is visible from here on
     pdl_wait();
-    pdl_trigger();
 
     // the grid is a multiple of the channel blocks: a CTA keeps one block
     const int nt = static_cast<int>(blockIdx.x) % a.n_ntiles, mt0 = static_cast<int>(blockIdx.x) / a.n_ntiles;
@@ -1130,6 +1128,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_gather_kernel(const Args a)
         epilogue_role<XMODE, WSRC>(a, sh, tmem, mt0, nt);
     } else if (warp == kMmaWarp) {
         const Chunks ck = make_chunks<WSRC>(a, sh, nt);
+        // the next kernel in the stream may launch now; it waits for this one before it
+        // touches memory
+        pdl_trigger();
         mma_role<XMODE, WSRC>(a, smem, sh, tmem, mt0, ck);
     } else if (WSRC == kWCopy) {
         copy_filters(a, smem, sh, mt0, nt);
