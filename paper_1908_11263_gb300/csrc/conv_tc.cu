@@ -173,7 +173,7 @@ __device__ __forceinline__ bool nt_run_ends(const TcArgs &a, int t)
 // Warp-converged bounded wait (all lanes poll; the result is warp-uniform).
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int *status)
 {
-    return mbar_wait_warp(bar, parity, status);
+    return mbar_wait_warp_timed(bar, parity, status);
 }
 
 // ---------------------------------------------------------------- u8 / sub-byte -> fp16 (8 channels)
