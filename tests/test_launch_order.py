@@ -42,7 +42,10 @@ def test_kernels_are_found():
     assert {"conv_win_kernel", "conv_gather_kernel", "conv_tc_prep_kernel", "pack_kernel", "unpack_kernel",
             "maxpool_vec_kernel", "linear_smem_kernel"} <= set(KERNELS)
     # the exemption holds only while that kernel is launched plainly
-    assert re.search(r"conv_tc_prep_kernel<B><<<", KERNELS["conv_tc_prep_kernel"][0])
+    text = KERNELS["conv_tc_prep_kernel"][0]
+    start = text.index("cudaError_t launch_conv_tc_prep(")
+    launch = text[start:text.index("\n}\n", start)]
+    assert "<<<" in launch and "cudaLaunchKernelEx" not in launch and "launch_pdl" not in launch
 
 
 @pytest.mark.parametrize("name", sorted(k for k, (_, body) in KERNELS.items() if TRIGGER.search(body)))
