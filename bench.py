@@ -607,10 +607,10 @@ def run_sweep(args):
             t_kernel = graph_time(lambda i: prepared(xs[i % nsets], out=ys[i % nsets], stream=stream), count, 3)
         qnn.device_status(stream)
         tk = t_kernel if t_kernel is not None else t_call
-        opbits = qnn.mma_operand_bits(desc)
-        kernel = {qnn.ALGO_TC_WINDOW: "window", qnn.ALGO_TC_GENERAL: "general", 0: "direct"}[qnn.tc_kernel(desc)]
-        line = {"sweep": config, "layer": layer.name, "algo": "tensorcore" if algo == qnn.ALGO_TENSORCORE else "direct",
-                "kernel": kernel,
+        # the kernel that us_kernel times: the prepared launch where there is one
+        kid, opbits = qnn.kernel(desc, prepared=t_kernel is not None)
+        line = {"sweep": config, "layer": layer.name, "algo": "tensorcore" if opbits else "direct",
+                "kernel": kernel_name(kid),
                 "mma_operands": {16: "fp16", 8: "e4m3", 0: "none (CUDA cores)"}[opbits],
                 "macs": layer.macs, "gmacs_call": round(layer.macs / t_call / 1e9, 1), "us_call": round(t_call * 1e6, 3),
                 "gmacs_kernel": round(layer.macs / tk / 1e9, 1), "us_kernel": round(tk * 1e6, 3),
@@ -658,11 +658,19 @@ def run_sweep(args):
         conv_line("3", key, layer, wl, lid)
     run_cifar_pipeline(layers, layer_tensors, graph_time, stream, dev)
     run_pool_linear(graph_time, stream, dev, pk)
-    run_binary(graph_time, stream, dev)
+    run_binary(graph_time, stream, dev, roof)
 
 
-def run_binary(graph_time, stream, dev):
-    """INT-1 (XNOR / popcount) convolution on the benchmark layer's shape, against the popcount roof."""
+def kernel_name(kid):
+    """A qnn.kernel() answer as text."""
+    from paper_1908_11263_gb300 import qnn
+    name = {qnn.KERNEL_DIRECT: "direct", qnn.KERNEL_COUNT: "count", qnn.KERNEL_WINDOW: "window",
+            qnn.KERNEL_GENERAL: "general", qnn.KERNEL_GATHER: "gather"}[kid & 0xF]
+    return name + (", whole rows" if kid & qnn.KERNEL_ROWS else "") + (", stacked" if kid & qnn.KERNEL_STACKED else "")
+
+
+def run_binary(graph_time, stream, dev, roof):
+    """INT-1 convolution on the benchmark layer's shape, against the roof of the kernel that runs it."""
     import torch
     from paper_1908_11263_gb300 import qnn
     rng = np.random.default_rng(12)
@@ -676,14 +684,17 @@ def run_binary(graph_time, stream, dev):
     t = graph_time(lambda i: qnn.conv_binary(xs[i % nsets], wt, tau, pad=1, out=ys[i % nsets], stream=stream), 200, 3)
     qnn.device_status(stream)
     macs = n * h * w * m * k * k * c
-    achieved = macs / t / 1e12
-    peak = POPC_TPS * 32
-    print(json.dumps({"sweep": "int1", "layer": "binary conv3x3_16x16x32_to_64 n512 (XNOR/popcount)",
+    kid, opbits = qnn.kernel(qnn.conv_desc(n, h, w, c, m, k, k, 1, 1, 1))
+    if opbits:  # tensor cores
+        roofline = roof(2.0 * macs, xbytes + ybytes + m * k * k * c // 8 + 4 * m, t, opbits)
+    else:
+        peak = POPC_TPS * 32
+        roofline = {"bound": "alu", "achieved": round(macs / t / 1e12, 2), "peak": round(peak, 1),
+                    "unit": "T binary MAC/s", "frac": round(macs / t / 1e12 / peak, 4),
+                    "peak_source": "measured popc rate x 32 bits per count"}
+    print(json.dumps({"sweep": "int1", "layer": "binary conv3x3_16x16x32_to_64 n512", "kernel": kernel_name(kid),
                       "macs": macs, "us_kernel": round(t * 1e6, 3), "gmacs_kernel": round(macs / t / 1e9, 1),
-                      "roofline": {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 1),
-                                   "unit": "T binary MAC/s", "frac": round(achieved / peak, 4),
-                                   "peak_source": "measured popc rate x 32 bits per count"},
-                      "l2": f"rotating {nsets} buffer sets"}), flush=True)
+                      "roofline": roofline, "l2": f"rotating {nsets} buffer sets"}), flush=True)
 
 
 def run_pool_linear(graph_time, stream, dev, pk):

@@ -57,8 +57,8 @@ enum {
                                   that needs no workspace (reported as QNN_ALGO_DIRECT: at INT-8 the tensor-core
                                   gather kernel, else the CUDA-core kernel) */
     QNN_ALGO_DIRECT = 1,       /* CUDA-core kernel (dp4a), any stride / padding */
-    QNN_ALGO_TENSORCORE = 2,   /* tcgen05 implicit GEMM (the window kernel when its plan fits, else the
-                                  general one); QNN_EUNSUPPORTED when neither fits the shape */
+    QNN_ALGO_TENSORCORE = 2,   /* tcgen05 kernels with preparable filters (the window kernel when its plan fits, else
+                                  the gather or the general kernel); QNN_EUNSUPPORTED when none fits the shape */
     QNN_ALGO_TC_WINDOW = 3,    /* the window kernel only: stride 1, m <= 128, INT-8 with c a multiple of 8
                                   or INT-4/INT-2 with c a multiple of 32, c <= 64 (INT-8) or 128 (sub-byte),
                                   kh, kw <= 8; one launch per call, filters read in place */
@@ -231,29 +231,48 @@ qnn_status qconv_hwc_thresholds(const qnn_conv_desc *d, const void *x, const voi
  *   thresholds  device int32 [m], 4-byte aligned
  *   y           device, NHWC bits [n][oh][ow][m / 8 bytes]
  *
- * Runs on CUDA cores (XNOR and population count).  QNN_EUNSUPPORTED when bits
- * is not 1 or c, m are not multiples of 8.
+ * Runs on the window tensor-core kernel (+1 / -1 values as e4m3) where that fits
+ * and x and w are 16-byte aligned, else on CUDA cores (XNOR and population
+ * count).  QNN_EUNSUPPORTED when bits is not 1 or c, m are not multiples of 8.
  */
 qnn_status qconv_hwc_binary(const qnn_conv_desc *d, const void *x, const void *w, const int32_t *thresholds,
                             void *y, void *stream);
 
-/* Which kernel qconv_hwc() would run for d: QNN_ALGO_DIRECT or QNN_ALGO_TENSORCORE;
- * negative qnn_status on invalid or unsupported descriptors. */
+/* Whether d's filters can be prepared: QNN_ALGO_TENSORCORE when they can (qconv_hwc_prepare
+ * and qconv_hwc_run take d, and qconv_hwc() may need a workspace), QNN_ALGO_DIRECT when not
+ * (qconv_hwc() runs a kernel that needs no workspace); negative qnn_status on invalid or
+ * unsupported descriptors.  qconv_hwc_kernel() names the kernel. */
 int32_t qconv_hwc_algo(const qnn_conv_desc *d);
 
-/* Which tensor-core kernel qconv_hwc() would run for d: QNN_ALGO_TC_WINDOW or
- * QNN_ALGO_TC_GENERAL; 0 when d selects the CUDA-core kernel; negative qnn_status
- * on invalid or unsupported descriptors. */
+/* Whose preparation and workspace rules d follows: the window kernel's (QNN_ALGO_TC_WINDOW) or
+ * the general kernel's (QNN_ALGO_TC_GENERAL); 0 when d's filters cannot be prepared; negative
+ * qnn_status on invalid or unsupported descriptors.  Layers with the general kernel's rules may
+ * run on another kernel: qconv_hwc_kernel() names it. */
 int32_t qconv_hwc_tc_kernel(const qnn_conv_desc *d);
 
-/* Operand format of the tensor-core MMAs qconv_hwc() would issue for d, so that a
- * caller can take the right tensor roof: 16 for fp16 operands (tcgen05 kind::f16,
- * the exact embedding of INT-8 and of sub-byte layers with c not a multiple of 32),
- * 8 for e4m3 operands (kind::f8f6f4, twice the fp16 rate per MMA; INT-4/INT-2 with
- * c a multiple of 32), 0 when d selects the CUDA-core kernel; negative qnn_status
- * on invalid or unsupported descriptors.  Not a paper concept: a query about this
- * library's kernel choice. */
+/* Operand format of d's prepared filters: 16 for fp16 (tcgen05 kind::f16, the exact
+ * embedding of INT-8 and of sub-byte layers with c not a multiple of 32), 8 for e4m3
+ * (kind::f8f6f4, twice the fp16 rate per MMA; INT-4/INT-2 with c a multiple of 32), 0 when
+ * d's filters cannot be prepared; negative qnn_status on invalid or unsupported
+ * descriptors.  Not a paper concept: a query about this library's kernel choice. */
 int32_t qconv_hwc_mma_operand_bits(const qnn_conv_desc *d);
+
+/* Which kernel a call launches for d on the current device, as QNN_KERNEL_* (with flags for the
+ * window kernel): qconv_hwc(), or with bits == 1 qconv_hwc_binary() on 16-byte aligned tensors
+ * (prepared == 0); qconv_hwc_run() (prepared != 0).  *operand_bits (may be NULL) receives the
+ * operand width of its tensor-core MMAs, so that a caller can take the right tensor roof: 16 (fp16),
+ * 8 (e4m3), or 0 for a CUDA-core kernel.  Negative qnn_status on invalid or unsupported
+ * descriptors, QNN_EUNSUPPORTED also for filters that cannot be prepared (prepared != 0). */
+enum {
+    QNN_KERNEL_DIRECT = 1,      /* CUDA cores, dp4a */
+    QNN_KERNEL_COUNT = 2,       /* CUDA cores, XNOR and population count (INT-1) */
+    QNN_KERNEL_WINDOW = 3,      /* window tensor-core kernel */
+    QNN_KERNEL_GENERAL = 4,     /* general tensor-core kernel */
+    QNN_KERNEL_GATHER = 5,      /* gather tensor-core kernel (INT-8) */
+    QNN_KERNEL_ROWS = 0x10,     /* flag: windows read as whole image rows, on the general kernel's workspace rules */
+    QNN_KERNEL_STACKED = 0x20   /* flag: tiles run across the images of the batch */
+};
+int32_t qconv_hwc_kernel(const qnn_conv_desc *d, int32_t prepared, int32_t *operand_bits);
 
 /* Size of the fixed scratch array behind qconv_hwc_noalloc(): 2 MiB. */
 enum { QNN_NOALLOC_SCRATCH_BYTES = 2097152 };

@@ -85,8 +85,8 @@ qnn_status check_conv(const qnn_conv_desc *d, ConvShape *s)
 // benchmark sweep), else the general tensor-core kernel; QNN_ALGO_TC_WINDOW and
 // QNN_ALGO_TC_GENERAL force one of them.  INT-8 layers that no prepared kernel
 // takes run on the gather kernel with the caller's filters (3 to 80 times as
-// fast as the CUDA-core kernel); they are reported as QNN_ALGO_DIRECT, need no
-// workspace and cannot be prepared.  One-shot calls of layers left to the general
+// fast as the CUDA-core kernel); qconv_hwc_algo() counts them as QNN_ALGO_DIRECT, as
+// they need no workspace and cannot be prepared.  One-shot calls of layers left to the general
 // kernel whose pixels are no whole 16-byte units run on the window kernel with
 // windows read as whole image rows (INT-2 staircase, 34 x 32 x 32 -> 16, batch
 // 1,453: 83.9 us, 200.9 on the general kernel);
@@ -149,11 +149,66 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
     return c;
 }
 
-// QNN_ALGO_DIRECT or QNN_ALGO_TENSORCORE (either tensor-core kernel), or a negative status.
+// QNN_ALGO_TENSORCORE (filters can be prepared) or QNN_ALGO_DIRECT (no workspace), or a negative status.
 int algo_of(const Choice &c)
 {
     if (c.kernel < 0) return c.kernel;
     return c.kernel == kDirect || c.kernel == kGather ? QNN_ALGO_DIRECT : QNN_ALGO_TENSORCORE;
+}
+
+// INT-1: the window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows), from
+// 128 products per output on: below that the counts are few (209 images of 7 x 20 x 32 -> 88, 1 x 1: 6.8 us
+// with counts, 11.5 there; 299 of 30 x 28 x 64 -> 104, 1 x 1: 21.7 and 20.6; 3 x 3 layers of 32 channels 26.4 and 9.7).
+WinPlan plan_binary(const ConvShape &s)
+{
+    const bool many = static_cast<long long>(s.kh) * s.kw * s.c >= 128;
+    WinPlan p = many ? plan_conv_win_batch(s) : WinPlan{};
+    p.ok = p.ok && p.nch_max == 1;
+    return p;
+}
+
+// Descriptor of an INT-1 layer.
+qnn_status check_binary(const qnn_conv_desc *d, ConvShape *s)
+{
+    if (!d || d->struct_size != sizeof(qnn_conv_desc)) return QNN_EINVAL;
+    if (d->n < 0 || d->h <= 0 || d->w <= 0 || d->c <= 0 || d->m <= 0 || d->kh <= 0 || d->kw <= 0) return QNN_EINVAL;
+    if (d->stride_h <= 0 || d->stride_w <= 0 || d->pad_h < 0 || d->pad_w < 0) return QNN_EINVAL;
+    if (d->h + 2 * d->pad_h < d->kh || d->w + 2 * d->pad_w < d->kw) return QNN_EINVAL;
+    if (d->bits != 1 || d->c % 8 || d->m % 8) return QNN_EUNSUPPORTED;
+    if (static_cast<long long>(d->kh) * d->kw * d->c >= (1ll << 31)) return QNN_EUNSUPPORTED;
+    *s = ConvShape{};
+    s->n = d->n; s->h = d->h; s->w = d->w; s->c = d->c; s->m = d->m; s->kh = d->kh; s->kw = d->kw;
+    s->sh = d->stride_h; s->sw = d->stride_w; s->ph = d->pad_h; s->pw = d->pad_w; s->bits = 1;
+    s->oh = (d->h + 2 * d->pad_h - d->kh) / d->stride_h + 1;
+    s->ow = (d->w + 2 * d->pad_w - d->kw) / d->stride_w + 1;
+    return QNN_OK;
+}
+
+// qconv_hwc_kernel's answers.
+int32_t window_kernel(const WinPlan &p) { return QNN_KERNEL_WINDOW | (p.period ? QNN_KERNEL_STACKED : 0); }
+
+int32_t launched_kernel(const Choice &c, bool prepared, int32_t *operand_bits)
+{
+    switch (c.kernel) {
+        case kWindow:
+            *operand_bits = c.wplan.fp8 ? 8 : 16;
+            return window_kernel(c.wplan);
+        case kRows:
+            if (prepared) break;
+            *operand_bits = c.wplan.fp8 ? 8 : 16;
+            return window_kernel(c.wplan) | QNN_KERNEL_ROWS;
+        case kWide:
+            *operand_bits = 16;
+            return QNN_KERNEL_GATHER;
+        case kDirect:
+        case kGather:
+            if (prepared) return -QNN_EUNSUPPORTED;
+            *operand_bits = c.kernel == kGather ? 16 : 0;
+            return c.kernel == kGather ? QNN_KERNEL_GATHER : QNN_KERNEL_DIRECT;
+        default: break;
+    }
+    *operand_bits = c.plan.fp8 ? 8 : 16;
+    return QNN_KERNEL_GENERAL;
 }
 
 qnn_status from_cuda(cudaError_t e) { return e == cudaSuccess ? QNN_OK : QNN_ECUDA; }
@@ -261,6 +316,28 @@ int32_t qconv_hwc_mma_operand_bits(const qnn_conv_desc *d)
     if (c.kernel == kWindow) return c.wplan.fp8 ? 8 : 16;
     if (c.kernel == kGeneral || c.kernel == kWide || c.kernel == kRows) return c.plan.fp8 ? 8 : 16;
     return 0;
+}
+
+int32_t qconv_hwc_kernel(const qnn_conv_desc *d, int32_t prepared, int32_t *operand_bits)
+{
+    ConvShape s;
+    int32_t bits = 0, kernel;
+    if (d && d->struct_size == sizeof(qnn_conv_desc) && d->bits == 1) {
+        const qnn_status st = check_binary(d, &s);
+        if (st != QNN_OK) return -static_cast<int32_t>(st);
+        if (prepared) return -QNN_EUNSUPPORTED;
+        const WinPlan p = plan_binary(s);
+        bits = p.ok ? 8 : 0;
+        kernel = p.ok ? window_kernel(p) : QNN_KERNEL_COUNT;
+    } else {
+        const qnn_status st = check_conv(d, &s);
+        if (st != QNN_OK) return -static_cast<int32_t>(st);
+        const Choice c = choose(d, s);
+        if (c.kernel < 0) return c.kernel;
+        kernel = launched_kernel(c, prepared != 0, &bits);
+    }
+    if (kernel >= 0 && operand_bits) *operand_bits = bits;
+    return kernel;
 }
 
 qnn_status qconv_hwc_prepare(const qnn_conv_desc *d, const void *w, const int32_t *bias, const int16_t *kappa,
@@ -441,25 +518,13 @@ qnn_status qconv_hwc_thresholds(const qnn_conv_desc *d, const void *x, const voi
 qnn_status qconv_hwc_binary(const qnn_conv_desc *d, const void *x, const void *w, const int32_t *thresholds, void *y,
                             void *stream)
 {
-    if (!d || d->struct_size != sizeof(qnn_conv_desc)) return QNN_EINVAL;
-    if (d->n < 0 || d->h <= 0 || d->w <= 0 || d->c <= 0 || d->m <= 0 || d->kh <= 0 || d->kw <= 0) return QNN_EINVAL;
-    if (d->stride_h <= 0 || d->stride_w <= 0 || d->pad_h < 0 || d->pad_w < 0) return QNN_EINVAL;
-    if (d->h + 2 * d->pad_h < d->kh || d->w + 2 * d->pad_w < d->kw) return QNN_EINVAL;
-    if (d->bits != 1 || d->c % 8 || d->m % 8) return QNN_EUNSUPPORTED;
-    if (static_cast<long long>(d->kh) * d->kw * d->c >= (1ll << 31)) return QNN_EUNSUPPORTED;
+    ConvShape s;
+    const qnn_status st = check_binary(d, &s);
+    if (st != QNN_OK) return st;
     if (!w || !thresholds || (d->n > 0 && (!x || !y))) return QNN_EINVAL;
     if (!aligned(thresholds, 4)) return QNN_EALIGN;
-    ConvShape s{};
-    s.n = d->n; s.h = d->h; s.w = d->w; s.c = d->c; s.m = d->m; s.kh = d->kh; s.kw = d->kw;
-    s.sh = d->stride_h; s.sw = d->stride_w; s.ph = d->pad_h; s.pw = d->pad_w; s.bits = 1;
-    s.oh = (d->h + 2 * d->pad_h - d->kh) / d->stride_h + 1;
-    s.ow = (d->w + 2 * d->pad_w - d->kw) / d->stride_w + 1;
-    // The window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows), from
-    // 128 products per output on: below that the counts are few (209 images of 7 x 20 x 32 -> 88, 1 x 1: 6.8 us
-    // with counts, 11.5 there; 299 of 30 x 28 x 64 -> 104, 1 x 1: 21.7 and 20.6; 3 x 3 layers of 32 channels 26.4 and 9.7)
-    const bool many = static_cast<long long>(s.kh) * s.kw * s.c >= 128;
-    const WinPlan wplan = many ? plan_conv_win_batch(s) : WinPlan{};
-    if (wplan.ok && wplan.nch_max == 1 && aligned(x, 16) && aligned(w, 16)) {
+    const WinPlan wplan = plan_binary(s);
+    if (wplan.ok && aligned(x, 16) && aligned(w, 16)) {
         ConvParams p{};
         p.x = static_cast<const uint8_t *>(x);
         p.w = static_cast<const uint8_t *>(w);

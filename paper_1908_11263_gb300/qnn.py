@@ -23,11 +23,14 @@ QNN_OK, QNN_EINVAL, QNN_EUNSUPPORTED, QNN_EALIGN, QNN_ECUDA, QNN_ETIMEOUT, QNN_E
 QNN_ESCRATCH = 7
 NOALLOC_SCRATCH_BYTES = 2 << 20  # QNN_NOALLOC_SCRATCH_BYTES
 ALGO_AUTO, ALGO_DIRECT, ALGO_TENSORCORE, ALGO_TC_WINDOW, ALGO_TC_GENERAL = 0, 1, 2, 3, 4
+# qconv_hwc_kernel: the kernel, and flags of the window kernel
+KERNEL_DIRECT, KERNEL_COUNT, KERNEL_WINDOW, KERNEL_GENERAL, KERNEL_GATHER = 1, 2, 3, 4, 5
+KERNEL_ROWS, KERNEL_STACKED = 0x10, 0x20
 
 EXPORTED = ("qconv_hwc_workspace_size", "qconv_hwc", "qconv_hwc_prepare", "qconv_hwc_run", "qconv_hwc_algo", "qlinear", "qmaxpool", "pack_subbyte",
             "unpack_subbyte", "qnn_device_status", "qnn_status_string", "qnn_version", "qconv_hwc_noalloc",
             "qnn_selftest_wait_timeout", "qconv_hwc_thresholds", "qconv_hwc_binary", "qconv_hwc_pool2", "qconv_hwc_pool2_run",
-            "qconv_hwc_mma_operand_bits", "qconv_hwc_tc_kernel")
+            "qconv_hwc_mma_operand_bits", "qconv_hwc_tc_kernel", "qconv_hwc_kernel")
 
 
 class QnnError(RuntimeError):
@@ -89,6 +92,8 @@ def load(build_if_missing: bool = False):
         lib.qconv_hwc_mma_operand_bits.restype = I32
         lib.qconv_hwc_tc_kernel.argtypes = [DP]
         lib.qconv_hwc_tc_kernel.restype = I32
+        lib.qconv_hwc_kernel.argtypes = [DP, I32, ctypes.POINTER(I32)]
+        lib.qconv_hwc_kernel.restype = I32
         lib.qlinear.argtypes = [I32, I32, I32, P, P, P, P, P]
         lib.qlinear.restype = I32
         lib.qmaxpool.argtypes = [I32] * 7 + [P, P, P]
@@ -201,8 +206,8 @@ def conv_algo(desc: ConvDesc) -> int:
 
 
 def tc_kernel(desc: ConvDesc) -> int:
-    """The tensor-core kernel qconv_hwc() runs for this descriptor: ALGO_TC_WINDOW or
-    ALGO_TC_GENERAL (0 for the CUDA-core kernel)."""
+    """Whose preparation and workspace rules this descriptor follows: ALGO_TC_WINDOW or
+    ALGO_TC_GENERAL (0: its filters cannot be prepared)."""
     r = load().qconv_hwc_tc_kernel(ctypes.byref(desc))
     if r < 0:
         raise QnnError(-r, "qconv_hwc_tc_kernel")
@@ -210,12 +215,23 @@ def tc_kernel(desc: ConvDesc) -> int:
 
 
 def mma_operand_bits(desc: ConvDesc) -> int:
-    """Operand width of the tensor-core MMAs for this descriptor: 16 (fp16, kind::f16),
-    8 (e4m3, kind::f8f6f4) or 0 (CUDA-core kernel)."""
+    """Operand width of this descriptor's prepared filters: 16 (fp16, kind::f16), 8 (e4m3,
+    kind::f8f6f4) or 0 (they cannot be prepared)."""
     r = load().qconv_hwc_mma_operand_bits(ctypes.byref(desc))
     if r < 0:
         raise QnnError(-r, "qconv_hwc_mma_operand_bits")
     return r
+
+
+def kernel(desc: ConvDesc, prepared: bool = False) -> tuple[int, int]:
+    """The kernel a call launches for this descriptor (conv_hwc, or conv_binary at bits 1; with
+    `prepared` PreparedConv's), KERNEL_* with flags, and the operand width of its MMAs (16, 8, or 0
+    on CUDA cores)."""
+    bits = ctypes.c_int32(0)
+    r = load().qconv_hwc_kernel(ctypes.byref(desc), int(prepared), ctypes.byref(bits))
+    if r < 0:
+        raise QnnError(-r, "qconv_hwc_kernel")
+    return r, bits.value
 
 
 _workspaces: dict = {}
