@@ -157,11 +157,13 @@ int algo_of(const Choice &c)
 }
 
 // INT-1: the window kernel on +1 / -1 values where it fits (stride 1, c a multiple of 32, whole 16-byte rows), from
-// 128 products per output on: below that the counts are few (209 images of 7 x 20 x 32 -> 88, 1 x 1: 6.8 us
-// with counts, 11.5 there; 299 of 30 x 28 x 64 -> 104, 1 x 1: 21.7 and 20.6; 3 x 3 layers of 32 channels 26.4 and 9.7).
+// 6144 products per pixel on.  Its time goes with the pixels, the counts' with the pixels times kh kw c m: 36 images
+// of 38 x 20 x 128 -> 40, 1 x 1 (5120), take 6.1 us with counts and 7.8 there; 352 of 18 x 28 x 128 -> 8 5.0 and
+// 11.9; 14 of 32 x 40 x 64 -> 96 (6144) 8.3 and 7.2; 22 of 10 x 16 x 64 -> 112 (7168) 9.2 and 6.5; the 3 x 3 layer of
+// 32 -> 64 at batch 512 26.4 and 9.7.
 WinPlan plan_binary(const ConvShape &s)
 {
-    const bool many = static_cast<long long>(s.kh) * s.kw * s.c >= 128;
+    const bool many = static_cast<long long>(s.kh) * s.kw * s.c * s.m >= 6144;
     WinPlan p = many ? plan_conv_win_batch(s) : WinPlan{};
     p.ok = p.ok && p.nch_max == 1;
     return p;
