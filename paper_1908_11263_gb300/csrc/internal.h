@@ -117,7 +117,7 @@ struct WinPlan {
 // period: tiles run across the images of the batch, that many rows each (s.h + s.ph, or one more; s.oh at most).
 WinPlan plan_conv_win(const ConvShape &s, bool rows = false, int period = 0);
 // The plan to launch: with stacked images where that saves every SM a tile (each
-// takes the same time, whatever its rows), else without.  Both have the same
+// takes the same time, whatever its rows) and enough of them, else without.  Both have the same
 // prepared image.  Batch 256 of 56 x 56 x 64 -> 64, 3 x 3: 66.4 us, 74.6 without;
 // CIFAR-shaped network at batch 1,024 (its 8 x 8 layer): 85.6 us, 90.1 without.
 WinPlan plan_conv_win_batch(const ConvShape &s, bool rows = false);

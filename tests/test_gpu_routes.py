@@ -60,3 +60,16 @@ def test_binary(shape, kernel):
     qnn.device_status()
     check_guard(buf)
     assert first_mismatch(out.cpu().numpy().reshape(-1), want) is None
+
+
+# (n, h, w, c, m, k, pad, bits, stacked): a round saved of a few (short INT-8 filters keep the plain form), of many
+@pytest.mark.parametrize("n,h,w,c,m,k,pad,bits,stacked", [
+    (2048, 14, 14, 32, 64, 3, 1, 8, False), (1003, 57, 8, 16, 32, 3, 1, 8, False), (691, 45, 8, 32, 16, 1, 0, 8, False),
+    (2048, 14, 14, 32, 64, 3, 1, 4, True), (256, 56, 56, 64, 64, 3, 1, 8, True), (1024, 8, 8, 32, 64, 5, 2, 8, True),
+    (331, 7, 12, 32, 24, 3, 1, 8, True), (366, 44, 8, 16, 104, 3, 1, 8, True), (512, 16, 16, 32, 64, 3, 1, 8, False)])
+def test_stacked_line(n, h, w, c, m, k, pad, bits, stacked):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("rounds of 152 blocks")
+    d = qnn.conv_desc(n, h, w, c, m, k, k, 1, pad, bits)
+    for prepared in (False, True):
+        assert qnn.kernel(d, prepared)[0] == (STACKED if stacked else WINDOW)
