@@ -139,12 +139,8 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
         }
     } else if (d->algo != QNN_ALGO_TENSORCORE) {
         // layers that no stride-1 kernel takes: the gather kernel on the caller's filters
-        // (a few products per output, and few outputs: the CUDA-core kernel has no pipeline to fill; 7 images of
-        // 37 x 18 x 3 -> 160, 1 x 1 stride 2, take it 3.6 us, the gather kernel 6.0)
-        const long long k = static_cast<long long>(s.kh) * s.kw * s.c;
-        const bool tiny = k <= 8 && k * s.n * s.oh * s.ow * s.m <= (4ll << 20);
-        if (!tiny) c.gplan = plan_conv_gather(s, 0, device_sm_count());
-        c.kernel = c.gplan.ok ? kGather : kDirect;
+        c.gplan = plan_conv_gather(s, 0, device_sm_count());
+        c.kernel = c.gplan.ok && !direct_beats_gather(c.gplan, s, device_sm_count()) ? kGather : kDirect;
     }
     return c;
 }

@@ -122,6 +122,27 @@ GatherPlan plan_conv_gather(const ConvShape &s, int w_rows, int sms)
     return p;
 }
 
+// The CUDA-core kernel has no pipeline to fill: a few loads per output, and few
+// outputs, are done there before the gather kernel's first tile is.  Both times in
+// microseconds as measured over 370 random small layers (each within 8 % of the
+// CUDA-core kernel's, 15 % of the gather kernel's); of those no choice is more than
+// 18 % slower than the other kernel.  50 images of 60 x 29 x 3 -> 23, 1 x 1: 8.7 us
+// on CUDA cores, 22.0 here; 36 of 10 x 58 x 1 -> 11, 3 x 3: 6.6 and 10.3; 12 of 41 x 5 x 4
+// -> 13, 3 x 4 stride 2: 11.2 and 5.5.
+bool direct_beats_gather(const GatherPlan &p, const ConvShape &s, int sms)
+{
+    const bool words = s.c % 4 == 0;  // four channels per load
+    const long long taps = static_cast<long long>(s.kh) * s.kw, loads = taps * (words ? s.c / 4 : s.c);
+    if (loads > 20) return false;
+    const double waves = static_cast<double>(s.n) * s.oh * s.ow * ((s.m + 7) / 8) / (1024.0 * sms);
+    const double filled = loads * std::min(s.m, 8) / 8.0;  // a thread's outputs, of eight
+    const double direct = words ? 2.45 + 0.32 * taps + 0.45 * filled + waves * (2.7 + 0.31 * filled)
+                                : 2.50 + 0.20 * taps + 0.14 * filled + waves * (3.2 + 0.10 * filled);
+    const double rounds = static_cast<double>((p.mtiles + p.mstep - 1) / p.mstep);
+    const double gather = 4.5 + 0.9 * rounds * p.nxs + 1.4 * (rounds * p.ncols / 64 - 1);
+    return direct < gather;
+}
+
 namespace {
 
 using namespace gather;

@@ -153,6 +153,8 @@ struct GatherPlan {
 // w_rows: filters per block of the workspace that launch_conv_tc_prep wrote
 // (with chunks = 0); 0: packed filters as the caller keeps them.
 GatherPlan plan_conv_gather(const ConvShape &s, int w_rows, int sms);
+// Whether the CUDA-core kernel takes a layer with the caller's filters (w_rows = 0) in less time.
+bool direct_beats_gather(const GatherPlan &plan, const ConvShape &s, int sms);
 cudaError_t launch_conv_gather(const GatherPlan &plan, const ConvShape &s, const ConvParams &p, cudaStream_t st);
 // wpack, chan: the filters and records launch_conv_tc_prep wrote
 cudaError_t launch_conv_gather_prepared(const GatherPlan &plan, const ConvShape &s, const uint8_t *x, uint8_t *y,

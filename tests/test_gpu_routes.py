@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_1908_11263_gb300 import qnn
 
-from gpu_util import check_guard, dev, first_mismatch, guarded_output
+from gpu_util import check_guard, conv_gpu, conv_oracle, dev, first_mismatch, guarded_output
 
 pytestmark = pytest.mark.gpu
 
@@ -73,3 +73,58 @@ def test_stacked_line(n, h, w, c, m, k, pad, bits, stacked):
     d = qnn.conv_desc(n, h, w, c, m, k, k, 1, pad, bits)
     for prepared in (False, True):
         assert qnn.kernel(d, prepared)[0] == (STACKED if stacked else WINDOW)
+
+
+def _layer(seed, n, h, w, c, m, kh, kw):
+    """Random INT-8 layer whose outputs spread over the byte range; one channel's constants need 64 bits."""
+    rng = np.random.default_rng(seed)
+    x, wt = rng.integers(0, 256, size=(n, h, w, c)), rng.integers(-128, 128, size=(m, kh, kw, c))
+    bias = rng.integers(-4096, 4097, size=m).astype(np.int32)
+    kappa = rng.integers(-64, 65, size=m).astype(np.int16)
+    lam = rng.integers(-(1 << 15), (1 << 15) + 1, size=m).astype(np.int32)
+    shift = int(np.ceil(np.log2(max(1.0, 2 * np.sqrt(kh * kw * c) * 147 * 74 * 33 / 255))))
+    shifts = (shift + rng.integers(-1, 2, size=m)).astype(np.uint8)
+    kappa[0], lam[0] = 32767, (1 << 31) - 1
+    return x, wt, bias, kappa, lam, shifts
+
+
+DIRECT, GATHER = qnn.KERNEL_DIRECT, qnn.KERNEL_GATHER
+# (n, h, w, c, m, kh, kw, stride, pad): the smallest layer and three channel blocks on packed filters; few loads per
+# output and many outputs, words and bytes, on either side of the line to the CUDA cores
+SMALL = [
+    ((1, 1, 1, 21, 1, 1, 1, 1, 0), GATHER),
+    ((1, 5, 3, 21, 300, 1, 1, 1, 3), GATHER),
+    ((1, 7, 9, 3, 5, 3, 3, 2, 1), GATHER),
+    ((12, 41, 5, 4, 13, 3, 4, 2, 1), GATHER),
+    ((12, 40, 44, 16, 100, 2, 2, 2, 0), GATHER),
+    ((1, 1, 1, 1, 1, 1, 1, 1, 0), DIRECT),
+    ((50, 60, 29, 3, 23, 1, 1, 1, 0), DIRECT),
+    ((36, 10, 58, 1, 11, 3, 3, 1, 1), DIRECT),
+    ((8, 42, 16, 16, 5, 1, 1, 3, 0), DIRECT),
+    ((5, 9, 11, 8, 2, 2, 2, 2, 1), DIRECT),
+]
+
+
+@pytest.mark.parametrize("shape,kernel", SMALL, ids=lambda v: _name(v) if isinstance(v, tuple) else str(v))
+def test_small_layers(shape, kernel):
+    n, h, w, c, m, kh, kw, stride, pad = shape
+    assert qnn.kernel(qnn.conv_desc(n, h, w, c, m, kh, kw, stride, pad))[0] == kernel
+    x, wt, bias, kappa, lam, shifts = _layer(sum(shape), n, h, w, c, m, kh, kw)
+    want = conv_oracle(x, wt, bias, kappa, lam, shifts, 0, 8, (stride, stride), (pad, pad))
+    got = conv_gpu(x, wt, bias, kappa, lam, shifts, 0, 8, (stride, stride), (pad, pad), qnn.ALGO_AUTO)
+    assert first_mismatch(got, want) is None, first_mismatch(got, want)
+
+
+@pytest.mark.parametrize("per_channel", [True, False])
+def test_gather_long_shifts(per_channel):
+    """Shifts from 0 to 62 in the gather kernel's 32-bit form (kappa small enough for it)."""
+    n, h, w, c, m = 2, 9, 9, 24, 64
+    assert qnn.kernel(qnn.conv_desc(n, h, w, c, m, 3, 3, 2, 1))[0] == GATHER
+    x, wt, bias, _, lam, _ = _layer(7, n, h, w, c, m, 3, 3)
+    kappa = np.where(np.arange(m) % 2, 1, -1).astype(np.int16)
+    lam = np.where(np.arange(m) % 3, 100, -100).astype(np.int32)
+    for shift in (0, 31, 32, 40, 62):
+        shifts = ((np.arange(m) + shift) % 63).astype(np.uint8) if per_channel else None
+        want = conv_oracle(x, wt, bias, kappa, lam, shifts, shift, 8, (2, 2), (1, 1))
+        got = conv_gpu(x, wt, bias, kappa, lam, shifts, shift, 8, (2, 2), (1, 1), qnn.ALGO_AUTO)
+        assert first_mismatch(got, want) is None, (shift, first_mismatch(got, want))
