@@ -358,8 +358,7 @@ qnn_status qconv_hwc_prepare(const qnn_conv_desc *d, const void *w, const int32_
     }
     st = check_workspace(plan, workspace, workspace_bytes);
     if (st != QNN_OK) return st;
-    return from_cuda(launch_conv_tc_prep(plan, s, p, workspace, static_cast<cudaStream_t>(stream),
-                                         c.kernel == kWide ? 0 : plan.nchunks));
+    return from_cuda(launch_conv_tc_prep(plan, s, p, workspace, static_cast<cudaStream_t>(stream)));
 }
 
 qnn_status qconv_hwc_run(const qnn_conv_desc *d, const void *x, void *y, const void *workspace,
@@ -383,9 +382,9 @@ qnn_status qconv_hwc_run(const qnn_conv_desc *d, const void *x, void *y, const v
     st = check_workspace(c.plan, workspace, workspace_bytes);
     if (st != QNN_OK) return st;
     if (c.kernel == kWide)
-        return from_cuda(launch_conv_gather_prepared(
-            c.gplan, s, static_cast<const uint8_t *>(x), static_cast<uint8_t *>(y), workspace,
-            static_cast<const uint8_t *>(workspace) + conv_tc_chan_offset(c.plan), static_cast<cudaStream_t>(stream)));
+        return from_cuda(launch_conv_gather_prepared(c.gplan, c.plan, s, static_cast<const uint8_t *>(x),
+                                                     static_cast<uint8_t *>(y), workspace,
+                                                     static_cast<cudaStream_t>(stream)));
     return from_cuda(launch_conv_tc_run(c.plan, s, static_cast<const uint8_t *>(x), static_cast<uint8_t *>(y),
                                         workspace, static_cast<cudaStream_t>(stream), false));
 }
@@ -416,12 +415,10 @@ qnn_status qconv_hwc(const qnn_conv_desc *d, const void *x, const void *w, const
         ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
                      d->shift, static_cast<uint8_t *>(y)};
         if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-        cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, c.kernel == kWide ? 0 : plan.nchunks);
+        cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs);
         if (e != cudaSuccess) return QNN_ECUDA;
         if (c.kernel == kWide)
-            return from_cuda(launch_conv_gather_prepared(
-                c.gplan, s, p.x, p.y, workspace,
-                static_cast<const uint8_t *>(workspace) + conv_tc_chan_offset(plan), cs));
+            return from_cuda(launch_conv_gather_prepared(c.gplan, plan, s, p.x, p.y, workspace, cs));
         return from_cuda(launch_conv_tc_run(plan, s, p.x, p.y, workspace, cs, true));
     }
     if (s.n == 0) return QNN_OK;
@@ -456,7 +453,7 @@ qnn_status qconv_hwc_pool2(const qnn_conv_desc *d, const void *x, const void *w,
     st = check_workspace(plan, workspace, workspace_bytes);
     if (st != QNN_OK) return st;
     if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-    cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, plan.nchunks);
+    cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs);
     if (e == cudaSuccess) e = launch_conv_tc_run(plan, s, p.x, p.y, workspace, cs, true);
     return from_cuda(e);
 }
@@ -505,7 +502,7 @@ qnn_status qconv_hwc_thresholds(const qnn_conv_desc *d, const void *x, const voi
         st = check_workspace(plan, workspace, workspace_bytes);
         if (st != QNN_OK) return st;
         if (c.kernel == kRows) return from_cuda(launch_conv_win(c.wplan, s, p, cs));
-        cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs, plan.nchunks);
+        cudaError_t e = launch_conv_tc_prep(plan, s, p, workspace, cs);
         if (e == cudaSuccess) e = launch_conv_tc_run(plan, s, p.x, p.y, workspace, cs, true);
         return from_cuda(e);
     }
@@ -562,7 +559,7 @@ qnn_status qconv_hwc_noalloc(const qnn_conv_desc *d, const void *x, const void *
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     ConvParams p{static_cast<const uint8_t *>(x), static_cast<const uint8_t *>(w), bias, kappa, lambda, shifts,
                  d->shift, static_cast<uint8_t *>(y)};
-    cudaError_t e = launch_conv_tc_prep(plan, s, p, scratch, cs, plan.nchunks);
+    cudaError_t e = launch_conv_tc_prep(plan, s, p, scratch, cs);
     if (e == cudaSuccess) e = launch_conv_tc_run(plan, s, p.x, p.y, scratch, cs, true);
     return from_cuda(e);
 }

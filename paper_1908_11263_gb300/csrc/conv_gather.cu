@@ -238,16 +238,17 @@ cudaError_t launch_conv_gather(const GatherPlan &p, const ConvShape &s, const Co
     return p.aligned ? launch_one<true, kIm2col, kWConvert>(a, p, st) : launch_one<false, kIm2col, kWConvert>(a, p, st);
 }
 
-cudaError_t launch_conv_gather_prepared(const GatherPlan &p, const ConvShape &s, const uint8_t *x, uint8_t *y,
-                                        const void *wpack, const void *chan, cudaStream_t st)
+cudaError_t launch_conv_gather_prepared(const GatherPlan &p, const TcPlan &prep, const ConvShape &s, const uint8_t *x,
+                                        uint8_t *y, const void *workspace, cudaStream_t st)
 {
     if (s.n == 0) return cudaSuccess;
     Args a = gather_args(p, s);
     if (!a.status) return cudaErrorInvalidSymbol;
     a.x = x;
     a.y = y;
-    a.wpack = static_cast<const uint8_t *>(wpack);
-    a.chan = static_cast<const int4 *>(chan);
+    a.wpack = static_cast<const uint8_t *>(workspace);
+    a.chan = reinterpret_cast<const int4 *>(a.wpack + conv_tc_chan_offset(prep));
+    a.preload = static_cast<uint32_t>(prep.nchunks) * kMagic;
     // the sums of |w| stand behind the records (by 64-channel group: the flat window's stages)
     a.wabs = p.flat && p.nxs <= kMaxAbs ? reinterpret_cast<const int32_t *>(a.chan + 2 * p.n_ntiles * p.w_rows) : nullptr;
     return p.flat ? launch_one<true, kFlat, kWCopy>(a, p, st) : launch_one<true, kIm2col, kWCopy>(a, p, st);

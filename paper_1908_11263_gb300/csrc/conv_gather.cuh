@@ -110,6 +110,7 @@ struct Args {
     int shift;
     const uint8_t *wpack;   // kWCopy: fp16 filters [n-tile][K / 8][w_rows][8]
     const int4 *chan;       // kWCopy: [2][n-tiles * w_rows] records
+    uint32_t preload;       // kWCopy: what the records subtract from the sums for the general kernel's pre-loads
     const int32_t *wabs;    // kWCopy: sums of |w| [filter][kMaxAbs], or null
     int h, w_, c, m, kh, kw, sh, sw, ph, pw, oh, ow;
     int row_c;              // input bytes per image row (w * c)
@@ -874,6 +875,9 @@ __device__ __forceinline__ bool channel_record(const Args &a, Shared *sh, int nt
         if (has) {
             r0 = a.chan[o];
             r1 = a.chan[a.n_ntiles * a.w_rows + o];
+            // (the records are modulo 2^32: lam2 = beta * kappa + lambda)
+            r0.x = static_cast<int32_t>(static_cast<uint32_t>(r0.x) + a.preload * static_cast<uint32_t>(r0.y));
+            r1.x = static_cast<int32_t>(static_cast<uint32_t>(r1.x) + a.preload);
         }
         return true;
     }

@@ -1218,8 +1218,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(const TcArgs a)
 // [0, 2^Q-1]); mode "clamp" when the saturation bounds allow a 32-bit form.
 // The kernel lets the convolution that follows it start at once (that kernel
 // waits for these results only where it reads them).
-// GROUPS: for the gather kernel, with the sums of |w| by 64-channel group.
-template <int BITS, bool GROUPS = false>
+// INT-8: also the sums of |w| by 64-channel group, for the gather kernel (which
+// takes the pre-load out of the records again), so that one preparation serves
+// both kernels.
+template <int BITS>
 __global__ void __launch_bounds__(256) conv_tc_prep_kernel(const uint8_t *w, const int32_t *bias, const int16_t *kappa,
                                                            const int32_t *lambda, const uint8_t *shifts, int shift,
                                                            int m, int mp, int kh, int kw, int c, int c_pad, int k_pad,
@@ -1260,33 +1262,46 @@ __global__ void __launch_bounds__(256) conv_tc_prep_kernel(const uint8_t *w, con
         }
     };
     // (consecutive lanes: consecutive channels and slots)
-    if constexpr (!GROUPS) {
+    if constexpr (BITS != 8) {
         for (int tap = 0; tap < taps; ++tap)
             for (int cc = lane; cc < c_pad; cc += 32) place(tap, cc, value(tap, cc));
     } else {
-        // The gather kernel: 64 channels at a time (its stages), all taps of them, and
-        // the group's sum of |w|.  The loads of four taps go out together: one-shot calls of
-        // 13 images of 16 x 16 x 128 -> 96, 5 x 5, take 44.5 us, 56.9 with one tap's at a time
-        // (51.6 on the general kernel), 46 of 4 x 4 x 192 -> 32, 3 x 3, 18.7 and 24.9 (21.6).
+        // 64 channels at a time (the gather kernel's stages), all taps of them, and the
+        // group's sum of |w|.  The loads of four steps go out together: one-shot calls of
+        // 13 images of 16 x 16 x 128 -> 96, 5 x 5, take 44.5 us, 56.9 with one step's at a time,
+        // 46 of 4 x 4 x 192 -> 32, 3 x 3, 18.7 and 24.9.
         constexpr int kBatch = 4;
-        for (int group = 0; group * 64 < c_pad; ++group) {
-            const int first_pos = pos, first_neg = neg, c0 = group * 64 + lane;
-            for (int tap = 0; tap < taps; tap += kBatch) {
-                int v[kBatch][2];
+        const int steps = (c_pad + 63) / 64 * taps;
+        int tap = 0, group = 0, before = 0;  // of the next step; the sum of |w| up to its group
+        for (int step = 0; step < steps; step += kBatch) {
+            int v[kBatch][2];
+            {
+                int t = tap, g = group;
 #pragma unroll
-                for (int b = 0; b < kBatch; ++b)
+                for (int b = 0; b < kBatch; ++b) {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) v[b][h] = tap + b < taps ? value(tap + b, c0 + h * 32) : 0;
-#pragma unroll
-                for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        if (tap + b < taps && c0 + h * 32 < c_pad) place(tap + b, c0 + h * 32, v[b][h]);
+                    for (int h = 0; h < 2; ++h) v[b][h] = step + b < steps ? value(t, g * 64 + lane + h * 32) : 0;
+                    if (++t == taps) {
+                        t = 0;
+                        ++g;
+                    }
+                }
             }
-            int abs = (pos - first_pos) - (neg - first_neg);
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) abs += __shfl_xor_sync(0xffffffffu, abs, d);
-            if (lane == 0 && group < kThrStride) thr_out[o * kThrStride + group] = abs;
+            for (int b = 0; b < kBatch; ++b) {
+                if (step + b >= steps) break;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (group * 64 + lane + h * 32 < c_pad) place(tap, group * 64 + lane + h * 32, v[b][h]);
+                if (++tap < taps) continue;
+                int abs = pos - neg - before;
+                before = pos - neg;
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) abs += __shfl_xor_sync(0xffffffffu, abs, d);
+                if (lane == 0 && group < kThrStride) thr_out[o * kThrStride + group] = abs;
+                tap = 0;
+                ++group;
+            }
         }
     }
 #pragma unroll
@@ -1571,7 +1586,7 @@ TcPlan plan_conv_tc(const ConvShape &s)
 size_t conv_tc_chan_offset(const TcPlan &plan) { return chan_offset(plan); }
 
 cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const ConvParams &p, void *workspace,
-                                cudaStream_t st, int chunks)
+                                cudaStream_t st)
 {
     uint16_t *wpack = static_cast<uint16_t *>(workspace);
     int4 *chan = reinterpret_cast<int4 *>(static_cast<uint8_t *>(workspace) + chan_offset(plan));
@@ -1579,12 +1594,12 @@ cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const Co
     int32_t *thr = reinterpret_cast<int32_t *>(chan + 2 * mp);
     auto prep = [&](auto kern) {
         kern<<<(mp + 7) / 8, 256, 0, st>>>(p.w, p.bias, p.kappa, p.lambda, p.shifts, p.shift, s.m, mp, s.kh, s.kw, s.c,
-                                           plan.c_pad, plan.k_pad, plan.nt, chunks, plan.fp8, wpack, chan, p.thresholds,
+                                           plan.c_pad, plan.k_pad, plan.nt, plan.nchunks, plan.fp8, wpack, chan, p.thresholds,
                                            thr);
         return cudaGetLastError();
     };
     switch (s.bits) {
-        case 8: return chunks == 0 ? prep(conv_tc_prep_kernel<8, true>) : prep(conv_tc_prep_kernel<8>);
+        case 8: return prep(conv_tc_prep_kernel<8>);
         case 4: return prep(conv_tc_prep_kernel<4>);
         default: return prep(conv_tc_prep_kernel<2>);
     }

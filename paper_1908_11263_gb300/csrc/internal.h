@@ -66,11 +66,10 @@ struct TcPlan {
 };
 
 TcPlan plan_conv_tc(const ConvShape &s);
-// chunks: accumulators per output whose pre-load the records remove
-// (plan.nchunks for conv_tc; 0 for the gather kernel, which has no pre-load and
-// gets the sums of |w| by filter and 64-channel group behind the records).
+// Filters and records (whose sums count plan.nchunks pre-loads); INT-8: behind the
+// records the sums of |w| by filter and 64-channel group, for the gather kernel.
 cudaError_t launch_conv_tc_prep(const TcPlan &plan, const ConvShape &s, const ConvParams &p, void *workspace,
-                                cudaStream_t st, int chunks);
+                                cudaStream_t st);
 // where launch_conv_tc_prep puts the compression records in the workspace
 size_t conv_tc_chan_offset(const TcPlan &plan);
 // after_prep: launched right after launch_conv_tc_prep on the same stream, so the
@@ -150,15 +149,14 @@ struct GatherPlan {
     uint32_t plane_x, stage_bytes, plane_w, item_w, off_x, off_bar, smem_bytes;
 };
 
-// w_rows: filters per block of the workspace that launch_conv_tc_prep wrote
-// (with chunks = 0); 0: packed filters as the caller keeps them.
+// w_rows: filters per block of the workspace that launch_conv_tc_prep wrote; 0: packed filters as the caller keeps them.
 GatherPlan plan_conv_gather(const ConvShape &s, int w_rows, int sms);
 // Whether the CUDA-core kernel takes a layer with the caller's filters (w_rows = 0) in less time.
 bool direct_beats_gather(const GatherPlan &plan, const ConvShape &s, int sms);
 cudaError_t launch_conv_gather(const GatherPlan &plan, const ConvShape &s, const ConvParams &p, cudaStream_t st);
-// wpack, chan: the filters and records launch_conv_tc_prep wrote
-cudaError_t launch_conv_gather_prepared(const GatherPlan &plan, const ConvShape &s, const uint8_t *x, uint8_t *y,
-                                        const void *wpack, const void *chan, cudaStream_t st);
+// workspace: the filters and records launch_conv_tc_prep wrote for `prep`
+cudaError_t launch_conv_gather_prepared(const GatherPlan &plan, const TcPlan &prep, const ConvShape &s, const uint8_t *x,
+                                        uint8_t *y, const void *workspace, cudaStream_t st);
 
 // ---- max-pool, fully connected, packing
 cudaError_t launch_maxpool(int n, int h, int w, int c, int k, int s, int bits, const uint8_t *x, uint8_t *y,
