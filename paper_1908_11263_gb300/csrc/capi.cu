@@ -102,16 +102,18 @@ struct Choice {
 
 // kGeneral, or kWide: the gather kernel on the filters and records that the
 // general kernel's preparation lays out (same workspace).
-int general_or_wide(Choice *c, const ConvShape &s)
+int general_or_wide(Choice *c, const ConvShape &s, bool one_shot)
 {
     if (c->plan.fp8) return kGeneral;
     c->gplan = plan_conv_gather(s, c->plan.nt, device_sm_count());
-    return c->gplan.ok ? kWide : kGeneral;
+    return c->gplan.ok && !general_beats_gather(c->gplan, c->plan, device_sm_count(), one_shot) ? kWide : kGeneral;
 }
 
 // The planners run in the order of preference and only as far as needed: a call
-// plans once (planning four times over cost a one-shot call about 3 us).
-Choice choose(const qnn_conv_desc *d, const ConvShape &s)
+// plans once (planning four times over cost a one-shot call about 3 us).  one_shot:
+// for a call that prepares its own filters; the choice between the general and
+// the gather kernel takes the preparation into account (same workspace).
+Choice choose(const qnn_conv_desc *d, const ConvShape &s, bool one_shot = false)
 {
     Choice c{};
     switch (d->algo) {
@@ -131,7 +133,7 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s)
     if (d->algo == QNN_ALGO_TC_WINDOW) return c;
     c.plan = plan_conv_tc(s);
     if (c.plan.ok) {
-        c.kernel = general_or_wide(&c, s);
+        c.kernel = general_or_wide(&c, s, one_shot);
         if (c.kernel == kGeneral) {
             // one-shot calls: the window kernel on windows read as whole image rows
             c.wplan = plan_conv_win_batch(s, true);
@@ -330,7 +332,7 @@ int32_t qconv_hwc_kernel(const qnn_conv_desc *d, int32_t prepared, int32_t *oper
     } else {
         const qnn_status st = check_conv(d, &s);
         if (st != QNN_OK) return -static_cast<int32_t>(st);
-        const Choice c = choose(d, s);
+        const Choice c = choose(d, s, prepared == 0);
         if (c.kernel < 0) return c.kernel;
         kernel = launched_kernel(c, prepared != 0, &bits);
     }
@@ -400,7 +402,7 @@ qnn_status qconv_hwc(const qnn_conv_desc *d, const void *x, const void *w, const
     if (!aligned(x, 16) || !aligned(y, 16)) return QNN_EALIGN;
     st = check_params(d, w, bias, kappa, lambda, shifts);
     if (st != QNN_OK) return st;
-    const Choice c = choose(d, s);
+    const Choice c = choose(d, s, true);
     if (c.kernel < 0) return static_cast<qnn_status>(-c.kernel);
     const TcPlan &plan = c.plan;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);

@@ -143,6 +143,41 @@ bool direct_beats_gather(const GatherPlan &p, const ConvShape &s, int sms)
     return direct < gather;
 }
 
+// The general kernel takes layers with prepared filters in less time where the
+// gather kernel runs im2col (a kernel of more than 16 taps) and 64 channels of
+// filters per step are streamed there, and where few filters stay resident there.
+// Times in microseconds as measured over 670 random layers (within 10 % each);
+// choosing by them leaves 22 us of the 493 that the gather kernel loses on 49 of the
+// layers.  25 images of 6 x 6 x 256 -> 16, 5 x 5: 68.0 us here, 47.0 there; 64 of 32 x
+// 32 x 64 -> 64, 7 x 7: 112.7 and 92.3; 15 of 7 x 7 x 256 -> 16, 3 x 3: 14.9 and 12.8; 14 of
+// 14 x 14 x 192 -> 280, 5 x 5: 53.2 and 56.6.  In one-shot calls the general kernel starts
+// beside the preparation, the gather kernel after it (2.1 us): 44 of 14 x 14 x 80 -> 8,
+// 3 x 3, take 12.1 us there and 15.4 here; 327 us lost on 365 layers become 11.
+bool general_beats_gather(const GatherPlan &p, const TcPlan &t, int sms, bool one_shot)
+{
+    if (t.b_resident && t.nt > 32) return false;
+    const double rounds = static_cast<double>((p.mtiles + p.mstep - 1) / p.mstep), ksteps = static_cast<double>(p.taps) * p.cgr;
+    double gather;
+    if (p.flat) {
+        gather = p.ncols <= 128   ? 3.1 + rounds * (3.1 + 0.060 * ksteps)
+                 : p.ncols == 192 ? 5.4 + rounds * (2.4 + 0.063 * ksteps)
+                                  : 4.7 + rounds * (2.7 + 0.084 * ksteps);
+    } else {
+        gather = p.ncols <= 64    ? 1.9 + rounds * (1.7 + 0.155 * ksteps)
+                 : p.ncols <= 128 ? 4.5 + rounds * (1.2 + 0.160 * ksteps)
+                                  : 5.5 + rounds * (1.0 + (p.resident ? 0.145 : 0.179) * ksteps);
+    }
+    const double tiles = static_cast<double>((t.total_tiles + sms - 1) / sms);
+    double general;
+    if (t.b_resident) {
+        general = 4.0 + tiles * (1.5 + 0.034 * t.mmas_per_tile + 0.6 * t.nslab);
+    } else {
+        const double mma = t.cs == 64 ? (t.nt == 128 ? 0.133 : 0.110) : t.cs == 32 ? 0.19 : 0.36;
+        general = 5.9 + tiles * (1.7 + mma * t.mmas_per_tile);
+    }
+    return general < gather + (one_shot ? 2.1 : 0.0);
+}
+
 namespace {
 
 using namespace gather;

@@ -153,6 +153,9 @@ struct GatherPlan {
 GatherPlan plan_conv_gather(const ConvShape &s, int w_rows, int sms);
 // Whether the CUDA-core kernel takes a layer with the caller's filters (w_rows = 0) in less time.
 bool direct_beats_gather(const GatherPlan &plan, const ConvShape &s, int sms);
+// Whether the general kernel takes a layer with prepared filters in less time
+// (one_shot: with its preparation).
+bool general_beats_gather(const GatherPlan &plan, const TcPlan &general, int sms, bool one_shot);
 cudaError_t launch_conv_gather(const GatherPlan &plan, const ConvShape &s, const ConvParams &p, cudaStream_t st);
 // workspace: the filters and records launch_conv_tc_prep wrote for `prep`
 cudaError_t launch_conv_gather_prepared(const GatherPlan &plan, const TcPlan &prep, const ConvShape &s, const uint8_t *x,

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_1908_11263_gb300 import qnn
 
-from gpu_util import check_guard, conv_gpu, conv_oracle, dev, first_mismatch, guarded_output
+from gpu_util import check_guard, conv_gpu, conv_oracle, dev, first_mismatch, guarded_output, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -128,3 +128,36 @@ def test_gather_long_shifts(per_channel):
         want = conv_oracle(x, wt, bias, kappa, lam, shifts, shift, 8, (2, 2), (1, 1))
         got = conv_gpu(x, wt, bias, kappa, lam, shifts, shift, 8, (2, 2), (1, 1), qnn.ALGO_AUTO)
         assert first_mismatch(got, want) is None, (shift, first_mismatch(got, want))
+
+
+GENERAL = qnn.KERNEL_GENERAL
+# (n, h, w, c, m, k, pad), prepared kernel, one-shot kernel: long kernels (more than 16 taps) of 64-channel steps, few
+# filters kept in shared memory, a preparation that only the general kernel starts beside, and the gather kernel's
+WIDE = [
+    ((2, 6, 6, 256, 16, 5, 2), GENERAL, GENERAL),
+    ((3, 7, 7, 192, 40, 7, 3), GENERAL, GENERAL),
+    ((2, 9, 8, 320, 88, 5, 2), GENERAL, GENERAL),
+    ((4, 8, 8, 80, 8, 3, 1), GATHER, GENERAL),
+    ((5, 7, 7, 256, 16, 3, 1), GENERAL, GENERAL),
+    ((2, 9, 8, 160, 88, 5, 2), GATHER, GATHER),
+    ((3, 14, 14, 128, 136, 3, 1), GATHER, GATHER),
+    ((2, 7, 6, 64, 192, 1, 0), GATHER, GATHER),
+]
+
+
+@pytest.mark.parametrize("shape,prepared,one_shot", WIDE, ids=lambda v: _name(v) if isinstance(v, tuple) else str(v))
+def test_wide_layers(shape, prepared, one_shot):
+    n, h, w, c, m, k, pad = shape
+    d = qnn.conv_desc(n, h, w, c, m, k, k, 1, pad)
+    assert (qnn.kernel(d, True)[0], qnn.kernel(d)[0]) == (prepared, one_shot)
+    x, wt, bias, kappa, lam, shifts = _layer(sum(shape), n, h, w, c, m, k, k)
+    want = conv_oracle(x, wt, bias, kappa, lam, shifts, 0, 8, (1, 1), (pad, pad))
+    got = conv_gpu(x, wt, bias, kappa, lam, shifts, 0, 8, (1, 1), (pad, pad), qnn.ALGO_AUTO)
+    assert first_mismatch(got, want) is None, first_mismatch(got, want)
+    conv = qnn.PreparedConv(to_dev(wt, torch.int8), to_dev(kappa, torch.int16), to_dev(lam, torch.int32), n=n, h=h, wd=w,
+                            bias=to_dev(bias, torch.int32), shifts=to_dev(shifts, torch.uint8), pad=pad)
+    out, buf = guarded_output(conv.out_shape)
+    conv(to_dev(x, torch.uint8), out=out)
+    qnn.device_status()
+    check_guard(buf)
+    assert first_mismatch(out.cpu().numpy().reshape(-1), want) is None
