@@ -134,8 +134,10 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s, bool one_shot = false)
     c.plan = plan_conv_tc(s);
     if (c.plan.ok) {
         c.kernel = general_or_wide(&c, s, one_shot);
-        if (c.kernel == kGeneral) {
-            // one-shot calls: the window kernel on windows read as whole image rows
+        // One-shot calls: the window kernel on windows read as whole image rows; at INT-8 from 33 of the general
+        // kernel's tiles on (2 images of 34 x 28 x 24 -> 112, 3 x 3, 16 tiles: 10.9 us on the window kernel, 10.2 there;
+        // 5 of 26 x 44 x 40 -> 16, 1 x 1, 45 tiles: 6.0 and 7.0).
+        if (c.kernel == kGeneral && (s.bits != 8 || c.plan.total_tiles > 32)) {
             c.wplan = plan_conv_win_batch(s, true);
             if (c.wplan.ok) c.kernel = kRows;
         }
