@@ -12,6 +12,7 @@ dimension counts bytes):
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -161,8 +162,8 @@ class _Layer:
     workspace it needs."""
     __slots__ = ("desc", "ref", "out_shape", "nbytes", "own_nbytes")
 
-    def __init__(self, n, h, w, c, m, kh, kw, stride, pad, bits, shift, algo):
-        self.desc = d = conv_desc(n, h, w, c, m, kh, kw, stride, pad, bits, shift, algo)
+    def __init__(self, n, h, w, c, m, kh, kw, stride_h, stride_w, pad_h, pad_w, bits, shift, algo):
+        self.desc = d = conv_desc(n, h, w, c, m, kh, kw, (stride_h, stride_w), (pad_h, pad_w), bits, shift, algo)
         self.ref = ctypes.byref(d)
         self.out_shape = (n, (h + 2 * d.pad_h - kh) // d.stride_h + 1, (w + 2 * d.pad_w - kw) // d.stride_w + 1,
                           m * bits // 8)
@@ -173,23 +174,17 @@ class _Layer:
             self.own_nbytes = 0 if self.nbytes and tc_kernel(d) == ALGO_TC_WINDOW else self.nbytes
 
 
-_layers: dict = {}
-
-
+@functools.lru_cache(maxsize=512, typed=True)
 def _layer(*sizes) -> _Layer:
-    """The _Layer of these sizes; the last few hundred are kept (they hold no tensors)."""
-    layer = _layers.get(sizes)
-    if layer is None:
-        layer = _Layer(*sizes)
-        if len(_layers) >= 512:
-            _layers.clear()
-        _layers[sizes] = layer
-    return layer
+    """The _Layer of these sizes; the last few hundred are kept (they hold no tensors).  By type as
+    well: 8.0 and 8 are equal keys, and the ABI refuses the one."""
+    return _Layer(*sizes)
 
 
 def _pair(v):
-    """A stride or padding as a tuple (dictionary keys take no lists)."""
-    return v if isinstance(v, int) else tuple(v)
+    """A stride or padding as two values."""
+    a, b = (v, v) if isinstance(v, int) else v
+    return a, b
 
 
 def workspace_size(desc: ConvDesc) -> int:
@@ -266,7 +261,7 @@ def conv_hwc(x, w, kappa, lam, *, bias=None, shifts=None, shift=0, bits=8, strid
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    layer = _layer(n, h, wd, cb * per, m, kh, kw, _pair(stride), _pair(pad), bits, shift, algo)
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, *_pair(stride), *_pair(pad), bits, shift, algo)
     if out is None:
         out = x.new_empty(layer.out_shape)
     else:
@@ -298,7 +293,7 @@ def conv_hwc_pool2(x, w, kappa, lam, *, bias=None, shifts=None, shift=0, bits=8,
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    layer = _layer(n, h, wd, cb * per, m, kh, kw, 1, _pair(pad), bits, shift, algo)
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, 1, 1, *_pair(pad), bits, shift, algo)
     _, oh, ow, mb = layer.out_shape
     if out is None:
         out = x.new_empty((n, oh // 2, ow // 2, mb))
@@ -329,7 +324,7 @@ def conv_hwc_thresholds(x, w, thresholds, *, bits, stride=1, pad=0, algo=ALGO_AU
         raise ValueError("x and w disagree on the channel count")
     if tuple(thresholds.shape) != (m, (1 << bits) - 1):
         raise ValueError(f"thresholds must have shape {(m, (1 << bits) - 1)}")
-    layer = _layer(n, h, wd, cb * per, m, kh, kw, _pair(stride), _pair(pad), bits, 0, algo)
+    layer = _layer(n, h, wd, cb * per, m, kh, kw, *_pair(stride), *_pair(pad), bits, 0, algo)
     if out is None:
         out = x.new_empty(layer.out_shape)
     else:
@@ -355,7 +350,7 @@ def conv_binary(x, w, thresholds, *, stride=1, pad=0, out=None, stream=None):
     m, kh, kw, cb2 = w.shape
     if cb != cb2:
         raise ValueError("x and w disagree on the channel count")
-    layer = _layer(n, h, wd, cb * 8, m, kh, kw, _pair(stride), _pair(pad), 1, 0, ALGO_AUTO)
+    layer = _layer(n, h, wd, cb * 8, m, kh, kw, *_pair(stride), *_pair(pad), 1, 0, ALGO_AUTO)
     if out is None:
         out = x.new_empty(layer.out_shape)
     else:
