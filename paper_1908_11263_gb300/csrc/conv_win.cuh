@@ -1131,6 +1131,12 @@ __device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile &e)
 {
     constexpr int CW = NT / 2;
     constexpr bool kCst = KIND == kEpiDirect || KIND == kEpiShifts;
+    // kEpiRec: every channel by compress_slow, which takes all forms, or the direct ones
+    // apart, which costs a branch per value (channels past 32 bits, 37 images of 31 x 40 x 16
+    // -> 120, 3 x 3: 33.4 us, 37.4 with the branch).  The kernels of up to 64 channels keep the
+    // branch: without it their code comes out such that layers that never get here are
+    // slower (256 of 56 x 56 x 64 -> 64, 3 x 3: 67.1 us instead of 66.1).
+    constexpr bool kOneForm = NT == 128;
     // kEpiShfl: the constants of channel col0 + c sit in lane c % 32 of set c / 32
     uint32_t my_lam2[2], my_kap[2], my_sh[2];
     if constexpr (KIND == kEpiShfl) {
@@ -1211,7 +1217,7 @@ __device__ __forceinline__ void epi_tile(const WinArgs &a, const EpiTile &e)
                                                 e.thr + (m0 + g0 + k) * (kThrStride / 4));
                         y1[k] = staircase<BITS>(static_cast<int32_t>(v1[g0 + k]), r0,
                                                 e.thr + (m0 + g0 + k) * (kThrStride / 4));
-                    } else if (r0.w == kModeDirect) {
+                    } else if (!kOneForm && r0.w == kModeDirect) {
                         y0[k] = static_cast<int32_t>(v0[g0 + k] * r0.y + r0.x) >> r0.z;
                         y1[k] = static_cast<int32_t>(v1[g0 + k] * r0.y + r0.x) >> r0.z;
                     } else {
