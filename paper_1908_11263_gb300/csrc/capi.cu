@@ -109,6 +109,20 @@ int general_or_wide(Choice *c, const ConvShape &s, bool one_shot)
     return c->gplan.ok && !general_beats_gather(c->gplan, c->plan, device_sm_count(), one_shot) ? kWide : kGeneral;
 }
 
+// Whether a one-shot layer left to the general kernel takes less time on the window kernel with whole-row windows.
+// INT-8: from 33 of the general kernel's tiles on (2 images of 34 x 28 x 24 -> 112, 3 x 3, 16 tiles: 10.9 us on the
+// window kernel, 10.2 there; 5 of 26 x 44 x 40 -> 16, 1 x 1, 45 tiles: 6.0 and 7.0).  Sub-byte: unless the images fill
+// the window kernel's tiles (twice the pixels) so badly that it has no fewer rounds of them, from three on, in layers of
+// up to 9 taps whose pixels' outputs are whole words or at most 64 filters (which the general kernel stores fast): 941
+// images of 38 x 20 x 32 -> 48, 3 x 3, INT-2: 67.7 and 44.5; 734 of 13 x 48 x 32 -> 120 51.1 and 71.1.
+bool rows_beat_general(const WinPlan &w, const TcPlan &t, const ConvShape &s)
+{
+    if (s.bits == 8) return t.total_tiles > 32;
+    const long long sms = device_sm_count(), rounds = (w.total_tiles + sms - 1) / sms;
+    return rounds < 3 || rounds < (t.total_tiles + sms - 1) / sms || s.kh * s.kw > 9 ||
+           (t.nt > 64 && s.m * s.bits % 32 != 0);
+}
+
 // The planners run in the order of preference and only as far as needed: a call
 // plans once (planning four times over cost a one-shot call about 3 us).  one_shot:
 // for a call that prepares its own filters; the choice between the general and
@@ -134,12 +148,10 @@ Choice choose(const qnn_conv_desc *d, const ConvShape &s, bool one_shot = false)
     c.plan = plan_conv_tc(s);
     if (c.plan.ok) {
         c.kernel = general_or_wide(&c, s, one_shot);
-        // One-shot calls: the window kernel on windows read as whole image rows; at INT-8 from 33 of the general
-        // kernel's tiles on (2 images of 34 x 28 x 24 -> 112, 3 x 3, 16 tiles: 10.9 us on the window kernel, 10.2 there;
-        // 5 of 26 x 44 x 40 -> 16, 1 x 1, 45 tiles: 6.0 and 7.0).
-        if (c.kernel == kGeneral && (s.bits != 8 || c.plan.total_tiles > 32)) {
+        if (c.kernel == kGeneral) {
+            // one-shot calls: the window kernel on windows read as whole image rows
             c.wplan = plan_conv_win_batch(s, true);
-            if (c.wplan.ok) c.kernel = kRows;
+            if (c.wplan.ok && rows_beat_general(c.wplan, c.plan, s)) c.kernel = kRows;
         }
     } else if (d->algo != QNN_ALGO_TENSORCORE) {
         // layers that no stride-1 kernel takes: the gather kernel on the caller's filters

@@ -161,3 +161,30 @@ def test_wide_layers(shape, prepared, one_shot):
     qnn.device_status()
     check_guard(buf)
     assert first_mismatch(out.cpu().numpy().reshape(-1), want) is None
+
+
+ROWS = qnn.KERNEL_WINDOW | qnn.KERNEL_ROWS
+# (n, h, w, c, m, k, bits): images that fill the tiles, badly, badly with few rounds, and badly with byte stores
+@pytest.mark.parametrize("n,h,w,c,m,k,bits,want", [
+    (734, 13, 48, 32, 120, 3, 2, ROWS), (941, 38, 20, 32, 48, 3, 2, GENERAL), (2, 29, 24, 32, 64, 3, 2, ROWS),
+    (529, 11, 36, 32, 120, 3, 2, ROWS), (53, 51, 20, 32, 40, 1, 2, GENERAL), (2, 34, 28, 24, 112, 3, 8, GENERAL),
+    (5, 26, 44, 40, 16, 1, 8, ROWS)])
+def test_whole_rows_line(n, h, w, c, m, k, bits, want):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("rounds of 152 blocks")
+    d = qnn.conv_desc(n, h, w, c, m, k, k, 1, k // 2, bits)
+    assert qnn.kernel(d)[0] & ~qnn.KERNEL_STACKED == want
+    assert qnn.kernel(d, prepared=True)[0] == GENERAL
+
+
+@pytest.mark.parametrize("n,h,w,m,want", [(120, 20, 20, 48, GENERAL), (90, 20, 36, 120, ROWS)])
+def test_whole_rows_parity(n, h, w, m, want):
+    """INT-2, 3 x 3, on either side of that line."""
+    assert qnn.kernel(qnn.conv_desc(n, h, w, 32, m, 3, 3, 1, 1, 2))[0] & ~qnn.KERNEL_STACKED == want
+    rng = np.random.default_rng(n + m)
+    x, wt = rng.integers(0, 4, size=(n, h, w, 32)), rng.integers(-2, 2, size=(m, 3, 3, 32))
+    kappa = rng.integers(-64, 65, size=m).astype(np.int16)
+    lam, bias = rng.integers(-500, 500, size=m).astype(np.int32), rng.integers(-30, 30, size=m).astype(np.int32)
+    want = conv_oracle(x, wt, bias, kappa, lam, None, 8, 2, (1, 1), (1, 1))
+    got = conv_gpu(x, wt, bias, kappa, lam, None, 8, 2, (1, 1), (1, 1), qnn.ALGO_AUTO)
+    assert first_mismatch(got, want) is None, first_mismatch(got, want)

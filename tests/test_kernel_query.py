@@ -64,7 +64,7 @@ def test_binary_line(c, m, k, want):
 
 @pytest.mark.parametrize("n,h,w,c,m,k,bits,rows", [(2, 34, 28, 24, 112, 3, 8, False), (1, 15, 32, 24, 64, 1, 8, False),
                                                    (5, 26, 44, 40, 16, 1, 8, True), (52, 15, 52, 56, 32, 3, 8, True),
-                                                   (2, 29, 24, 32, 64, 3, 2, True)])
+                                                   (2, 29, 32, 32, 64, 3, 2, True)])
 def test_whole_rows_line(n, h, w, c, m, k, bits, rows):
     """INT-8 layers of few tiles stay on the general kernel."""
     kernel, _ = qnn.kernel(qnn.conv_desc(n, h, w, c, m, k, k, 1, k // 2, bits))
