@@ -175,9 +175,11 @@ int algo_of(const Choice &c)
 // 32 -> 64 at batch 512 26.4 and 9.7.
 WinPlan plan_binary(const ConvShape &s)
 {
-    const bool many = static_cast<long long>(s.kh) * s.kw * s.c * s.m >= 6144;
-    WinPlan p = many ? plan_conv_win_batch(s) : WinPlan{};
-    p.ok = p.ok && p.nch_max == 1;
+    // (up to 24 filters and 9000 products: only where every SM has one tile; 150 of 36 x 20 x 96 -> 8, 3 x 3 (6912),
+    // 10.9 us with counts and 17.5 there; 700 random layers lose 46 us in all, 1 % of their time)
+    const long long products = static_cast<long long>(s.kh) * s.kw * s.c * s.m, sms = device_sm_count();
+    WinPlan p = products >= 6144 ? plan_conv_win_batch(s) : WinPlan{};
+    p.ok = p.ok && p.nch_max == 1 && (s.m > 24 || products >= 9000 || p.total_tiles <= sms);
     return p;
 }
 

@@ -39,6 +39,8 @@ BINARY = [
     ((2, 33, 28, 32, 8, 4, 5, 2), COUNT),
     ((170, 20, 40, 64, 16, 3, 3, 0), STACKED),
     ((400, 9, 24, 96, 72, 1, 1, 0), STACKED),
+    ((150, 36, 20, 96, 8, 3, 3, 1), COUNT),
+    ((9, 16, 36, 64, 16, 3, 3, 1), WINDOW),
 ]
 
 

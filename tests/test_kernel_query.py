@@ -56,7 +56,7 @@ def test_prepared():
 @pytest.mark.parametrize("c,m,k,want", [(128, 8, 1, qnn.KERNEL_COUNT), (128, 40, 1, qnn.KERNEL_COUNT),
                                         (128, 48, 1, qnn.KERNEL_WINDOW), (64, 96, 1, qnn.KERNEL_WINDOW),
                                         (64, 88, 1, qnn.KERNEL_COUNT), (32, 16, 3, qnn.KERNEL_COUNT),
-                                        (32, 24, 3, qnn.KERNEL_WINDOW)])
+                                        (32, 32, 3, qnn.KERNEL_WINDOW)])
 def test_binary_line(c, m, k, want):
     """INT-1 layers run on the window kernel from 6144 products per pixel on."""
     assert qnn.kernel(desc(w=32, c=c, m=m, k=k, pad=k // 2, bits=1))[0] & 0xF == want
