@@ -82,10 +82,11 @@ qnn_status check_conv(const qnn_conv_desc *d, ConvShape *s)
 // QNN_ALGO_TENSORCORE) take the window kernel when its plan fits the shape,
 // else, at INT-8 with c a multiple of 16, the gather kernel on prepared
 // filters (2.5 to 3 times as fast as the general kernel on the layers of the
-// benchmark sweep), else the general tensor-core kernel; QNN_ALGO_TC_WINDOW and
+// benchmark sweep) where general_beats_gather does not say otherwise, else the
+// general tensor-core kernel; QNN_ALGO_TC_WINDOW and
 // QNN_ALGO_TC_GENERAL force one of them.  INT-8 layers that no prepared kernel
 // takes run on the gather kernel with the caller's filters (3 to 80 times as
-// fast as the CUDA-core kernel); qconv_hwc_algo() counts them as QNN_ALGO_DIRECT, as
+// fast as the CUDA-core kernel; the smallest stay there, direct_beats_gather); qconv_hwc_algo() counts them as QNN_ALGO_DIRECT, as
 // they need no workspace and cannot be prepared.  One-shot calls of layers left to the general
 // kernel whose pixels are no whole 16-byte units run on the window kernel with
 // windows read as whole image rows (INT-2 staircase, 34 x 32 x 32 -> 16, batch

@@ -1,8 +1,9 @@
 // Quantized INT-8 HWC convolution on the sm_103a tensor cores with the output
 // channels along the MMA's rows and output pixels along its columns: the
-// gather kernel.  It serves every INT-8 layer that the window kernel's plan
-// does not take: more than 128 filters, many channels, any stride, padding,
-// channel count and alignment.
+// gather kernel.  It serves INT-8 layers that the window kernel's plan does not
+// take: more than 128 filters, many channels, any stride, padding, channel count
+// and alignment, except where the general kernel or the CUDA cores are faster
+// (general_beats_gather, direct_beats_gather).
 //
 // What it computes (Sec. III-B, Eq. 6; Sec. III-A): for every output pixel p
 // and channel o,
@@ -53,14 +54,14 @@
 // (no workspace; the compression constants are derived here as well); kWCopy:
 // bulk copies of the fp16 filters that conv_tc_prep_kernel laid out.
 //
-// Measured per call (was: general tensor-core kernel for the first three, CUDA
-// cores for the others): 28 x 28 x 128 -> 128 3 x 3, batch 64: 16.1 us (49.2);
-// 14 x 14 x 256 -> 256 3 x 3: 15.8 us (47.3); 14 x 14 x 256 -> 512 1 x 1: 12.1 us
-// (30.7); 56 x 56 x 64 -> 128 3 x 3 stride 2: 19.9 us (1,627); 33 x 45 x 20 -> 44
-// 3 x 3, batch 37: 16.9 us (70; 25.4 with a branch per word of an unaligned
-// granule).  The flat-window layers are bound by the MMA warp's issue (an item of
-// four N = 192 MMAs takes 550 cycles, 384 without any wait); im2col layers by the
-// latency of the producers' global loads.
+// Measured per launch (was: general tensor-core kernel for the first three, CUDA
+// cores for the others): 28 x 28 x 128 -> 128 3 x 3, batch 64: 16.8 us (49.5);
+// 14 x 14 x 256 -> 256 3 x 3: 16.4 us (48.0); 14 x 14 x 256 -> 512 1 x 1: 12.6 us
+// (30.7); 56 x 56 x 64 -> 128 3 x 3 stride 2: 20.2 us (1,637); 33 x 45 x 20 -> 44
+// 3 x 3, batch 37: 17.0 us (70; 25.4 with a branch per word of an unaligned
+// granule; 18.2 on new buffers in each call).  The flat-window layers are bound by
+// the MMA warp's issue (an item of four N = 192 MMAs takes 550 cycles, 384 without
+// any wait); im2col layers by the latency of the producers' global loads.
 //
 // Warp roles (one persistent CTA per SM, 18 warps):
 //   warps 0-7    producers: global memory -> registers -> staged fp16
@@ -1015,7 +1016,7 @@ __device__ __forceinline__ void epilogue_role(const Args &a, Shared *sh, uint32_
                 }
                 const int p0 = mt * a.ncols + col0 + b0;  // the block's first column
                 const int mine = XMODE == kFlat ? output_pixel<XMODE>(a, p0 + lane) : 0;
-// Lane i of four has words of four pixels' bytes of its channel; afterwards
+                // Lane i of four has words of four pixels' bytes of its channel; afterwards
                 // it has pixel i's bytes of the four channels.  All eight words go through
                 // each step together: one at a time, with its store, took 160 cycles each.
                 uint32_t w[8];
